@@ -6,12 +6,12 @@
 //   dL/dw_i  += (1 - T)/B * a_i G.(c_i - r)
 //   dL/da_i  += w_i (1 - T)/B G.(c_i - r) - T/(1 - a_i) G.(c_bg - r)
 // and through a_i = o_i exp(-q/2) (zero when the 0.99 clamp is active) to
-// o_i, the pixel mean and the conic.  All of these only need (A, B, T) of the
+// o_i, the pixel mean and the covariance.  All of these only need (A, B, T) of the
 // forward, so the backward is as order-independent as the forward.
 //
-//   k_raster_bwd      one CTA per tile, same blocks and culling as the
-//                     forward; per-Gaussian partials are reduced across the
-//                     warp and added to a per-Gaussian gradient record.
+//   k_raster_bwd      one warp per 8x8 block, lane = Gaussian: a lane sums its
+//                     Gaussian's partials over the block's pixels in registers
+//                     and adds them to a per-Gaussian gradient record.
 //   k_preprocess_bwd  one thread per Gaussian: recomputes the forward, chains
 //                     through the EWA covariance, projection, SH colour,
 //                     Eq. 3 weight and (warp-cooperatively) the Eq. 4 MLP.
@@ -25,71 +25,312 @@
 namespace mgs {
 namespace {
 
-constexpr int kBwdThreads = 64;   // raster backward: two warps per tile
-constexpr int kRedGroup = 8;      // candidates reduced together through shared memory
+constexpr int kBwdThreads = 128;  // raster backward: four warps per CTA, one 8x8 block each
+constexpr int kBwdWarps = kBwdThreads / 32;
+constexpr int kBwdRing = 64;      // candidate slots per warp (a power of two)
 constexpr int kGRec = 12;         // per-Gaussian raster gradient record
-// layout: dc(3), dw, do, dm(2), dK(3) [conic A, B, C], pad(2)
+// layout: dc(3), dw, do, dm(2), M(3), pad(2), with M the second moments of s =
+// -2 dL/dq in the whitened coordinates e = L^T (pixel - mean) of the inclusion
+// test: sum s e1^2, sum s e1 e2, sum s e2^2.  dL/dSigma_2D = L M L^T / 2 and
+// dL/dm = L sum(s e) then have no cancelling terms, which the moments of
+// (dx, dy) have for elongated Gaussians.
 
+typedef unsigned long long f2;    // two packed FP32 lanes: two adjacent pixels
+__device__ __forceinline__ f2 pk(float lo, float hi) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void upk(f2 v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ float hsum(f2 v) {
+    float lo, hi;
+    upk(v, lo, hi);
+    return lo + hi;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 sub2(f2 a, f2 b) {
+    f2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
 __device__ __forceinline__ float ex2f(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+__device__ __forceinline__ float rcpf(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// p[0..3] += (a, b, c, d), p 16-byte aligned, without a result
+__device__ __forceinline__ void red4(float *p, float a, float b, float c, float d) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c),
+                 "f"(d)
+                 : "memory");
+}
 
+// Shared memory of the rasteriser adjoint, per warp: the constants of the
+// block's 32 horizontal pixel pairs (pair 4 y + x / 2), and the candidate ring.
+//   px0 = {k_A G_r (2 pixels), k_A G_g (2)}, px1 = {k_A G_b (2), -k_A G.r (2)},
+//   px2 = {-T G.(c_bg - r) (2)}
+//   ring[0] = {m_x, m_y, l11, l21}, ring[1] = {l22, log2 o, 1 / o, w},
+//   ring[2] = {c_r, c_g, c_b, Gaussian index}
+struct BwdRaster {
+    float4 px0[kBwdWarps][32], px1[kBwdWarps][32];
+    float2 px2[kBwdWarps][32];
+    float4 ring[kBwdWarps][3][kBwdRing];
+};
+
+// How a batch treats the pixels: kFast (every constant finite, no opacity above
+// 0.99: an excluded pixel's alpha is 0 and so is everything it adds), kClamped
+// (some opacity above 0.99) and kGuarded (a non-finite weight, colour or pixel
+// constant: excluded pixels are skipped, so that they add nothing).
+enum BwdMode { kFast, kClamped, kGuarded };
+
+// One batch: lane = one candidate, looping over the warp's 8x8 block at (bx0,
+// by0); adds the candidate's ten partials to its gradient record.
+//   per pixel with q <= 9 (a = min(a_raw, 0.99), u = k_A (G.c - G.r)):
+//     dc  += w a k_A G       dw += a u
+//   and, where the clamp is inactive, with s = a (w u - T G.(c_bg - r) / (1 - a)):
+//     do  += s / o,  and s e1, s e2, s e1^2, s e1 e2, s e2^2 for the mean and
+//     covariance terms (e2 is the same for a row: its moments are taken row by row).
+template <int kMode>
+__device__ __forceinline__ void bwd_batch(const BwdRaster &sm, int warp, int slot, bool active,
+                                          int bx0, int by0, float *__restrict__ gG) {
+    const float4 *px0 = sm.px0[warp], *px1 = sm.px1[warp];
+    const float2 *px2 = sm.px2[warp];
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = make_float4(0.f, -INFINITY, 0.f, 0.f), c = a;
+    if (active) {
+        a = sm.ring[warp][0][slot];
+        b = sm.ring[warp][1][slot];
+        c = sm.ring[warp][2][slot];
+    }
+    const float my = a.y, l21 = a.w, l22 = b.x;
+    const f2 l11 = pk(a.z, a.z), lo = pk(b.y, b.y), w = pk(b.w, b.w);
+    const f2 c0 = pk(c.x, c.x), c1 = pk(c.y, c.y), c2 = pk(c.z, c.z);
+    const float kq = -0.72134752044448170f;  // -log2(e) / 2
+    const f2 kq2 = pk(kq, kq), one = pk(1.0f, 1.0f), mx = pk(a.x, a.x);
+    f2 dx[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        dx[j] = sub2(pk((float)(bx0 + 2 * j) + 0.5f, (float)(bx0 + 2 * j) + 1.5f), mx);
+    f2 sc0 = 0ull, sc1 = 0ull, sc2 = 0ull, sw = 0ull, m11 = 0ull;
+    float s0 = 0.f, se1 = 0.f, se2 = 0.f, m12 = 0.f, m22 = 0.f;
+#pragma unroll 2
+    for (int r = 0; r < 8; ++r) {
+        const float dy = __fsub_rn((float)(by0 + r) + 0.5f, my);
+        const float ldys = __fmul_rn(l21, dy);
+        const float e2 = __fmul_rn(l22, dy);
+        const float e2q = __fmul_rn(e2, e2);
+        const f2 ldy = pk(ldys, ldys), e2s = pk(e2q, e2q);
+        f2 r0 = 0ull, r1 = 0ull;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float4 p0 = px0[4 * r + j], p1 = px1[4 * r + j];
+            const float2 p2 = px2[4 * r + j];
+            const f2 e1 = fma2(l11, dx[j], ldy);
+            const f2 q = fma2(e1, e1, e2s);
+            const f2 g = fma2(q, kq2, lo);
+            float qa, qb, ga, gb;
+            upk(q, qa, qb);
+            upk(g, ga, gb);
+            float aa = ex2f(ga), ab = ex2f(gb);
+            const bool ia = qa <= 9.0f, ib = qb <= 9.0f;
+            bool ua = true, ub = true;   // clamp inactive
+            if constexpr (kMode != kFast) {
+                ua = aa < 0.99f;
+                ub = ab < 0.99f;
+                aa = fminf(aa, 0.99f);
+                ab = fminf(ab, 0.99f);
+            }
+            aa = ia ? aa : 0.0f;
+            ab = ib ? ab : 0.0f;
+            const f2 al = pk(aa, ab);
+            f2 k0 = pk(p0.x, p0.y), k1 = pk(p0.z, p0.w), k2 = pk(p1.x, p1.y);
+            f2 kr = pk(p1.z, p1.w), tg = pk(p2.x, p2.y);
+            if constexpr (kMode == kGuarded) {   // excluded pixels: all constants 0
+                k0 = pk(ia ? p0.x : 0.f, ib ? p0.y : 0.f);
+                k1 = pk(ia ? p0.z : 0.f, ib ? p0.w : 0.f);
+                k2 = pk(ia ? p1.x : 0.f, ib ? p1.y : 0.f);
+                kr = pk(ia ? p1.z : 0.f, ib ? p1.w : 0.f);
+                tg = pk(ia ? p2.x : 0.f, ib ? p2.y : 0.f);
+            }
+            sc0 = fma2(al, k0, sc0);
+            sc1 = fma2(al, k1, sc1);
+            sc2 = fma2(al, k2, sc2);
+            f2 u = fma2(k0, c0, fma2(k1, c1, fma2(k2, c2, kr)));
+            // 1 - a >= 0.01: the fast reciprocal is accurate to a few ulp
+            float na, nb;
+            upk(sub2(one, al), na, nb);
+            const f2 inv = pk(rcpf(na), rcpf(nb));
+            f2 s;
+            if constexpr (kMode == kGuarded) {
+                float u0, u1;
+                upk(u, u0, u1);
+                u = pk(ia ? u0 : 0.f, ib ? u1 : 0.f);   // a non-finite colour times 0
+                sw = fma2(al, u, sw);
+                float v0, v1;
+                upk(mul2(al, fma2(w, u, mul2(tg, inv))), v0, v1);
+                s = pk(ia && ua ? v0 : 0.f, ib && ub ? v1 : 0.f);
+            } else {
+                sw = fma2(al, u, sw);
+                s = mul2(al, fma2(w, u, mul2(tg, inv)));
+                if constexpr (kMode == kClamped) {
+                    float v0, v1;
+                    upk(s, v0, v1);
+                    s = pk(ua ? v0 : 0.f, ub ? v1 : 0.f);
+                }
+            }
+            const f2 sx = mul2(s, e1);
+            r0 = add2(r0, s);
+            r1 = add2(r1, sx);
+            m11 = fma2(sx, e1, m11);
+        }
+        const float t0 = hsum(r0), t1 = hsum(r1), t2 = e2 * t0;
+        s0 += t0;
+        se1 += t1;
+        se2 += t2;
+        m12 = fmaf(e2, t1, m12);
+        m22 = fmaf(e2, t2, m22);
+    }
+    if (!active) return;
+    // dL/dq = -s / 2 per pixel and q = e^T e with e = L^T (pixel - m): dq/dm = -2 L e
+    const float io = b.z;
+    float acc[10];
+    acc[0] = b.w * hsum(sc0);
+    acc[1] = b.w * hsum(sc1);
+    acc[2] = b.w * hsum(sc2);
+    acc[3] = hsum(sw);
+    acc[4] = s0 * io;
+    acc[5] = a.z * se1;
+    acc[6] = fmaf(l21, se1, l22 * se2);
+    acc[7] = hsum(m11);
+    acc[8] = m12;
+    acc[9] = m22;
+    float *rec = gG + (size_t)__float_as_uint(c.w) * kGRec;
+    if (acc[0] != 0.f || acc[1] != 0.f || acc[2] != 0.f || acc[3] != 0.f)
+        red4(rec, acc[0], acc[1], acc[2], acc[3]);
+    if (io > 0.0f) {   // o = 0: no gradient through alpha
+        if (acc[4] != 0.f || acc[5] != 0.f || acc[6] != 0.f || acc[7] != 0.f)
+            red4(rec + 4, acc[4], acc[5], acc[6], acc[7]);
+        if (acc[8] != 0.f || acc[9] != 0.f) red4(rec + 8, acc[8], acc[9], 0.f, 0.f);
+    }
+}
+
+// Rasteriser adjoint.  `splits` CTAs per tile, each taking an equal share of the
+// tile's list; warp w owns the 8x8 block at (8 (w % 2), 8 (w / 2)) and streams
+// the share on its own, 32 entries at a time (one per lane), testing them
+// against its block and queueing the candidates in its ring.  Every 32
+// candidates make a batch in which a lane holds one Gaussian and loops over
+// the block's 64 pixels, whose constants all lanes read from shared memory
+// by broadcast: the ten partials of a (Gaussian, block) are plain register
+// sums, so nothing is reduced across lanes, and the three 16-byte reductions
+// per (Gaussian, block) are the only other traffic.
+//
+// Bound: the FP32 FMA pipe (19 packed operations of two cycles each per pixel
+// pair, 0.36 ms for the pairs below) and issue.  Measured at 300k Gaussians,
+// 1296x840 (12 M (block, Gaussian) pairs): 0.67 ms, 0.54 G instructions, FMA
+// pipe 60 % busy.  The layout it replaced (lane = four pixels of a 16x8 block,
+// ten partials per candidate reduced through shared memory, ten scalar
+// atomics) took 1.85 ms and 1.52 G instructions; at 30k, 333x251 (336 tiles)
+// 0.27 against 0.06 ms, there also because the lists are split over CTAs.
+// Variants that were slower: 80 registers for six CTAs per SM (0.69 ms,
+// spills), pairs unrolled by two instead of four (0.78 ms).
 __global__ void __launch_bounds__(kBwdThreads) k_raster_bwd(RenderArgs args,
                                                             const float *__restrict__ dL,
                                                             const float *__restrict__ aux,
-                                                            float *__restrict__ gG) {
-    __shared__ float4 buf[2][4][32];
-    // per warp: the partials of up to kRedGroup candidates, row (k, e), column
-    // lane; rows padded to 36 floats so eight lanes reading eight rows with
-    // 16-byte loads hit distinct banks
-    __shared__ __align__(16) float red[2][kRedGroup * 10][36];
+                                                            float *__restrict__ gG, int splits) {
+    __shared__ BwdRaster sm;
     const DevCamera &cam = args.cam;
-    const int tile = (int)(args.tile_order[blockIdx.x] & kTileMask);
+    const int tile = (int)(args.tile_order[blockIdx.x / splits] & kTileMask);
+    const int split = blockIdx.x % splits;
     const int tx = tile % cam.tiles_x, ty = tile / cam.tiles_x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int bx0 = tx * kTile, by0 = ty * kTile + 8 * warp;
-    const int px0 = bx0 + 4 * (lane & 3);
-    const int py = by0 + (lane >> 2);
+    const int bx0 = tx * kTile + 8 * (warp & 1), by0 = ty * kTile + 8 * (warp >> 1);
     if (args.status->last_pairs > args.capacity) return;
+    const uint32_t t0 = args.tile_offsets[tile], t1 = args.tile_offsets[tile + 1];
+    const uint32_t share = ((t1 - t0 + 31) / 32 + splits - 1) / splits * 32;   // whole batches
+    const uint32_t start = min((uint64_t)t0 + (uint64_t)split * share, (uint64_t)t1);
+    const uint32_t end = min((uint64_t)start + share, (uint64_t)t1);
+    if (start >= end) return;
 
-    // per-pixel constants from the forward's (A, B, T) and dL/dC, with
-    // k_A = (1 - T) / B and r = A / B:  kG = k_A G,  kGr = k_A G.r,
-    // TGb = T G.(c_bg - r)  (all zero for pixels without coverage)
-    const int64_t HW = (int64_t)cam.width * cam.height;
-    float kG[4][3], kGr[4], TGb[4];
+    // this lane's pixel pair: constants from the forward's (A, B, T) and dL/dC,
+    // with k_A = (1 - T) / B and r = A / B (all zero without coverage)
+    bool finite = true;
+    {
+        const int64_t HW = (int64_t)cam.width * cam.height;
+        const int py = by0 + (lane >> 2), x0 = bx0 + 2 * (lane & 3);
+        float k[5][2];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int x = px0 + k;
-        kG[k][0] = kG[k][1] = kG[k][2] = kGr[k] = TGb[k] = 0.f;
-        if (x < cam.width && py < cam.height) {
-            const int64_t p = (int64_t)py * cam.width + x;
-            const float B = aux[3 * HW + p];
-            if (B > 0.0f) {
-                const float T = aux[4 * HW + p];
-                const float inv = 1.0f / B;
-                const float kA = (1.0f - T) * inv;
-                float G[3], r[3];
+        for (int h = 0; h < 2; ++h) {
 #pragma unroll
-                for (int ch = 0; ch < 3; ++ch) {
-                    G[ch] = dL[3 * p + ch];
-                    r[ch] = aux[ch * HW + p] * inv;
-                    kG[k][ch] = kA * G[ch];
+            for (int e = 0; e < 5; ++e) k[e][h] = 0.f;
+            if (x0 + h < cam.width && py < cam.height) {
+                const int64_t p = (int64_t)py * cam.width + x0 + h;
+                const float B = aux[3 * HW + p];
+                if (B > 0.0f) {
+                    const float T = aux[4 * HW + p];
+                    const float inv = 1.0f / B;
+                    const float kA = (1.0f - T) * inv;
+                    float G[3], r[3];
+#pragma unroll
+                    for (int ch = 0; ch < 3; ++ch) {
+                        G[ch] = dL[3 * p + ch];
+                        r[ch] = aux[ch * HW + p] * inv;
+                        k[ch][h] = kA * G[ch];
+                    }
+                    k[3][h] = -kA * (G[0] * r[0] + G[1] * r[1] + G[2] * r[2]);
+                    k[4][h] = -T * (G[0] * (args.bg[0] - r[0]) + G[1] * (args.bg[1] - r[1]) +
+                                    G[2] * (args.bg[2] - r[2]));
                 }
-                kGr[k] = kA * (G[0] * r[0] + G[1] * r[1] + G[2] * r[2]);
-                TGb[k] = T * (G[0] * (args.bg[0] - r[0]) + G[1] * (args.bg[1] - r[1]) +
-                              G[2] * (args.bg[2] - r[2]));
             }
+#pragma unroll
+            for (int e = 0; e < 5; ++e) finite &= isfinite(k[e][h]);
         }
+        sm.px0[warp][lane] = make_float4(k[0][0], k[0][1], k[1][0], k[1][1]);
+        sm.px1[warp][lane] = make_float4(k[2][0], k[2][1], k[3][0], k[3][1]);
+        sm.px2[warp][lane] = make_float2(k[4][0], k[4][1]);
     }
-    const uint32_t start = args.tile_offsets[tile];
-    const uint32_t end = args.tile_offsets[tile + 1];
-    const float bx = (float)bx0 + 8.0f, by = (float)by0 + 4.0f;
-    const float pyc = (float)py + 0.5f;
-    const float kq = -0.72134752044448170f;  // -log2(e) / 2
-    float4(*wb)[32] = buf[warp];
+    const bool px_finite = __all_sync(0xffffffffu, finite);
+    const float bx = (float)bx0 + 4.0f, by = (float)by0 + 4.0f;
+    const float kLogClamp = -0.014499569695115089f;   // log2(0.99)
+    float4(*ring)[kBwdRing] = sm.ring[warp];
 
+    int head = 0, count = 0;   // queued candidates: ring slots [head, head + count)
+    auto batch = [&](int n) {
+        const int slot = (head + lane) & (kBwdRing - 1);
+        const bool active = lane < n;
+        bool special = false, clamp = false;
+        if (active) {
+            const float4 b = ring[1][slot], c = ring[2][slot];
+            special = !(fabsf(b.w) + fabsf(c.x) + fabsf(c.y) + fabsf(c.z) < INFINITY);
+            clamp = !(b.y <= kLogClamp);
+        }
+        if (!px_finite || __any_sync(0xffffffffu, special))
+            bwd_batch<kGuarded>(sm, warp, slot, active, bx0, by0, gG);
+        else if (__any_sync(0xffffffffu, clamp))
+            bwd_batch<kClamped>(sm, warp, slot, active, bx0, by0, gG);
+        else
+            bwd_batch<kFast>(sm, warp, slot, active, bx0, by0, gG);
+        __syncwarp();
+    };
     // list entries two batches ahead, their records one batch ahead
     uint32_t gid_n = 0, gid_nn = 0;
     float4 a_n = make_float4(0.f, 0.f, 0.f, 0.f), b_n = a_n, c_n = a_n;
@@ -104,7 +345,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_raster_bwd(RenderArgs args,
         const uint32_t j = base + lane;
         const uint32_t gid = gid_n;
         const float4 a = a_n, b = b_n, c = c_n;
-        const bool cand = j < end && block_may_hit(a.x, a.y, a.z, a.w, b.x, bx, by, 7.5f, 3.5f);
+        const bool cand = j < end && block_may_hit(a.x, a.y, a.z, a.w, b.x, bx, by, 3.5f, 3.5f);
         if (j + 32 < end) {
             gid_n = gid_nn;
             a_n = __ldg(&args.rec[gid_n].a);
@@ -114,98 +355,30 @@ __global__ void __launch_bounds__(kBwdThreads) k_raster_bwd(RenderArgs args,
         if (j + 64 < end) gid_nn = __ldg(&args.gids[j + 64]);
         const unsigned bal = __ballot_sync(0xffffffffu, cand);
         if (cand) {
-            const int pos = __popc(bal & ((1u << lane) - 1u));
+            const int pos = (head + count + __popc(bal & ((1u << lane) - 1u))) & (kBwdRing - 1);
             const float w = -b.z, o = exp2f(b.y);
             const float iw = 1.0f / w;
-            wb[0][pos] = a;
-            // 1/o (0 when o = 0: no opacity gradient then)
-            wb[1][pos] = make_float4(b.x, b.y, o > 0.0f ? 1.0f / o : 0.0f, w);
-            // colour c = (-w c) / (-w); conic (A, B, C) = L L^T from the factors
-            wb[2][pos] = make_float4(-b.w * iw, -c.x * iw, -c.y * iw, a.z * a.z);
-            wb[3][pos] = make_float4(a.z * a.w, a.w * a.w + b.x * b.x, __uint_as_float(gid), 0.f);
+            ring[0][pos] = a;
+            // 1 / o (0 when o = 0: no opacity gradient then); colour c = (-w c) / (-w)
+            ring[1][pos] = make_float4(b.x, b.y, o > 0.0f ? 1.0f / o : 0.0f, w);
+            ring[2][pos] = make_float4(-b.w * iw, -c.x * iw, -c.y * iw, __uint_as_float(gid));
         }
         __syncwarp();
-        const int nc = __popc(bal);
-        for (int k0 = 0; k0 < nc; k0 += kRedGroup) {
-        const int ng = min(kRedGroup, nc - k0);
-        for (int k = k0; k < k0 + ng; ++k) {
-            const float4 cs0 = wb[0][k], cs1 = wb[1][k], cs2 = wb[2][k], cs3 = wb[3][k];
-            const float mx = cs0.x, my = cs0.y, l11 = cs0.z, l21 = cs0.w;
-            const float l22 = cs1.x, lo = cs1.y, io = cs1.z, w = cs1.w;
-            const float cr = cs2.x, cg = cs2.y, cb = cs2.z, cA = cs2.w, cB = cs3.x, cC = cs3.y;
-            // per pixel with q <= 9 (a = min(a_raw, 0.99), u = k_A (G.c - G.r)):
-            //   dc  += w a kG          dw += a u
-            // and, where the clamp is inactive, with s = a (w u - TGb / (1 - a)):
-            //   do  += s / o,  and s, s dx, s dx^2 for the mean and conic terms
-            // (dy is the same for the lane's four pixels)
-            float sc0 = 0.f, sc1 = 0.f, sc2 = 0.f, sw = 0.f;
-            float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-            const float dy = __fsub_rn(pyc, my);
-            const float ldy = __fmul_rn(l21, dy);
-            const float e2 = __fmul_rn(l22, dy);
-            const float e2s = __fmul_rn(e2, e2);
-#pragma unroll
-            for (int px = 0; px < 4; ++px) {
-                const float dx = __fsub_rn((float)(px0 + px) + 0.5f, mx);
-                const float e1 = __fmaf_rn(l11, dx, ldy);
-                const float q = __fmaf_rn(e1, e1, e2s);
-                if (!(q <= 9.0f)) continue;
-                const float araw = ex2f(__fmaf_rn(q, kq, lo));
-                const float al = fminf(araw, 0.99f);
-                sc0 = fmaf(al, kG[px][0], sc0);
-                sc1 = fmaf(al, kG[px][1], sc1);
-                sc2 = fmaf(al, kG[px][2], sc2);
-                const float u = fmaf(kG[px][0], cr, fmaf(kG[px][1], cg, fmaf(kG[px][2], cb, -kGr[px])));
-                sw = fmaf(al, u, sw);
-                if (araw < 0.99f) {
-                    // 1 - al > 0.01: the fast reciprocal division is accurate to a few ulp
-                    const float sa = al * fmaf(w, u, -__fdividef(TGb[px], 1.0f - al));
-                    s0 += sa;
-                    s1 = fmaf(sa, dx, s1);
-                    s2 = fmaf(sa * dx, dx, s2);
-                }
-            }
-            float acc[10];
-            acc[0] = w * sc0;
-            acc[1] = w * sc1;
-            acc[2] = w * sc2;
-            acc[3] = sw;
-            if (io > 0.0f) {
-                // dL/dq = -s / 2 per pixel; q = A dx^2 + 2 B dx dy + C dy^2 gives
-                // dq/dm = -2 (A dx + B dy, B dx + C dy) and dq/d(A, B, C) =
-                // (dx^2, 2 dx dy, dy^2)
-                acc[4] = s0 * io;
-                acc[5] = fmaf(cA, s1, cB * dy * s0);
-                acc[6] = fmaf(cB, s1, cC * dy * s0);
-                acc[7] = -0.5f * s2;
-                acc[8] = -dy * s1;
-                acc[9] = -0.5f * dy * dy * s0;
-            } else {
-                acc[4] = acc[5] = acc[6] = acc[7] = acc[8] = acc[9] = 0.f;
-            }
-#pragma unroll
-            for (int e = 0; e < 10; ++e) red[warp][(k - k0) * 10 + e][lane] = acc[e];
+        count += __popc(bal);
+        if (count >= 32) {
+            batch(32);
+            head = (head + 32) & (kBwdRing - 1);
+            count -= 32;
         }
-        __syncwarp();
-        // transposed reduction: lane r sums row r (one candidate's partial e over
-        // the 32 lanes) and adds it to that candidate's gradient record
-        for (int r = lane; r < ng * 10; r += 32) {
-            const float4 *row = reinterpret_cast<const float4 *>(red[warp][r]);
-            float sum = 0.f;
-#pragma unroll
-            for (int v = 0; v < 8; ++v) {
-                const float4 x = row[v];
-                sum += (x.x + x.y) + (x.z + x.w);
-            }
-            if (sum != 0.0f) {
-                const int k = k0 + r / 10;
-                atomicAdd(gG + (size_t)__float_as_uint(wb[3][k].z) * kGRec + (r % 10), sum);
-            }
-        }
-        __syncwarp();
-        }
-        __syncwarp();
     }
+    if (count > 0) batch(count);
+}
+
+// CTAs per tile of the rasteriser adjoint: images with few tiles split their
+// lists so that about ten CTAs per SM are in flight.
+int bwd_splits(int T, int sm_count) {
+    const int s = (10 * sm_count + T - 1) / T;
+    return s < 1 ? 1 : (s > 8 ? 8 : s);
 }
 
 // ---------------------------------------------------------------------------
@@ -562,12 +735,6 @@ __global__ void __launch_bounds__(kMlpThreads) k_preprocess_bwd(RenderArgs args,
             V0[j] = T0[0] * M[j] + T0[1] * M[3 + j] + T0[2] * M[6 + j];
             V1[j] = T1[0] * M[j] + T1[1] * M[3 + j] + T1[2] * M[6 + j];
         }
-        const float ca = V0[0] * V0[0] + V0[1] * V0[1] + V0[2] * V0[2] + 0.3f;
-        const float cbv = V0[0] * V1[0] + V0[1] * V1[1] + V0[2] * V1[2];
-        const float ccv = V1[0] * V1[0] + V1[1] * V1[1] + V1[2] * V1[2] + 0.3f;
-        const float det = ca * ccv - cbv * cbv;
-        const float idet = vis ? 1.0f / det : 0.f;
-        const float KA = ccv * idet, KB = -cbv * idet, KC = ca * idet;
         int am = 0;
         float smax = v[3];
         if (v[4] > smax) { smax = v[4]; am = 1; }
@@ -578,13 +745,19 @@ __global__ void __launch_bounds__(kMlpThreads) k_preprocess_bwd(RenderArgs args,
         const float gcol[3] = {up[0], up[1], up[2]}, gw = up[3], go = up[4];
         float dt[3] = {0.f, 0.f, 0.f}, ds[3] = {0.f, 0.f, 0.f}, dq[4] = {0.f, 0.f, 0.f, 0.f};
         float dP[3] = {0.f, 0.f, 0.f}, dY[12];
-        // conic -> Sigma_2D:  dSigma = -K Gk K, Gk = [[gA, gB/2], [gB/2, gC]]
-        const float G00 = up[7], G01 = 0.5f * up[8], G11 = up[9];
-        const float KG00 = KA * G00 + KB * G01, KG01 = KA * G01 + KB * G11;
-        const float KG10 = KB * G00 + KC * G01, KG11 = KB * G01 + KC * G11;
-        const float dS00 = -(KG00 * KA + KG01 * KB), dS01 = -(KG00 * KB + KG01 * KC);
-        const float dS11 = -(KG10 * KB + KG11 * KC);
-        const float ga = dS00, gb = 2.0f * dS01, gc = dS11;
+        // whitened second moments -> Sigma_2D:  dSigma = L M L^T / 2, with the
+        // forward's factors L = [[l11, 0], [l21, l22]]
+        float l11 = 0.f, l21 = 0.f, l22 = 0.f;
+        if (vis) {
+            const float4 ra = __ldg(&args.rec[i].a);
+            l11 = ra.z;
+            l21 = ra.w;
+            l22 = __ldg(&args.rec[i].b.x);
+        }
+        const float LM00 = l11 * up[7], LM01 = l11 * up[8];   // first row of L M
+        const float LM10 = l21 * up[7] + l22 * up[8], LM11 = l21 * up[8] + l22 * up[9];
+        const float ga = 0.5f * LM00 * l11, gb = LM00 * l21 + LM01 * l22;   // gb: twice dSigma_01
+        const float gc = 0.5f * (LM10 * l21 + LM11 * l22);
         float dV0[3], dV1[3];
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
@@ -828,7 +1001,8 @@ cudaError_t launch_backward(const RenderArgs &a, int sm_count, const float *dL_d
     const int T = a.cam.tiles_x * a.cam.tiles_y;
     cudaError_t e = cudaMemsetAsync(gG, 0, (size_t)a.n * kGRec * sizeof(float), stream);
     if (e != cudaSuccess) return e;
-    k_raster_bwd<<<T, kBwdThreads, 0, stream>>>(a, dL_drgb, aux, gG);
+    const int splits = bwd_splits(T, sm_count);
+    k_raster_bwd<<<T * splits, kBwdThreads, 0, stream>>>(a, dL_drgb, aux, gG, splits);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int blocks = pre_bwd_blocks(a.n, sm_count);
     const bool fp16 = a.precision == MGS_PREC_FP16;
