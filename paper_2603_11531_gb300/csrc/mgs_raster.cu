@@ -3,29 +3,43 @@
 //   A = sum_i c_i a_i w_i,  B = sum_i a_i w_i,  T = prod_i (1 - a_i)
 //   C = (1 - T) A / B + T c_bg          (foreground term 0 when B = 0)
 //
-// FP32 scenes (k_raster): one CTA per 16x16 tile, 64 threads, each thread
-// owning four horizontally adjacent pixels (two packed FP32x2 pairs).  Each
-// warp owns a 16x8 block and walks the tile's Gaussian list itself, testing
-// each entry against its block with a conservative bound (block_may_hit) and
-// compacting (ballot) the candidates before accumulating them in registers.
+// One CTA per 16x16 tile, four warps of 8x8 pixels; the four lanes of a quad
+// own one row of eight pixels.  Each warp walks the tile's Gaussian list itself,
+// testing each entry against its block with a conservative bound
+// (block_may_hit) and compacting (ballot) the candidates into a ring in shared
+// memory; the lanes of a quad take different candidates, and their sums are
+// added at the end.
 //
-// FP16-attribute scenes (k_raster_tc): four warps of 8x8 pixels per tile;
-// alpha is still computed, tested and multiplied into T in FP32 exactly as
-// above, but a_i w_i c_i and a_i w_i are summed on the tensor cores by
+// FP32 scenes (k_raster): packed FP32x2 arithmetic over pixel pairs, all sums
+// on the FMA pipe.
+//
+// FP16-attribute scenes (k_raster_tc): alpha is computed, tested and multiplied
+// into T in FP32 exactly as above (packed over two candidates), but a_i w_i c_i
+// and a_i w_i are summed on the tensor cores by
 // mma.sync (m16n8k8, FP16 operands, FP32 accumulation) with the weights split
 // into FP16 high and low parts, which leaves alpha's FP16 rounding (relative
 // 2^-12 per term) as the only extra error; tiles listing a Gaussian outside
 // the FP16 weight range take the FP32 code.
 //
-// No atomics, no sort: every pixel is owned by exactly one thread, and a
-// tile's list is accumulated in whatever order binning stored it.
+// No atomics, no sort: every pixel belongs to one quad, and a tile's list is
+// accumulated in whatever order binning stored it.
+//
+// The FMA sums stop updating T once it cannot matter: when every lane of a warp holds
+// a partial product of at most 2^-12 for each of its pixels, T <= 2^-48, so
+// 1 - T is 1 in FP32 and T c_bg is below 2^-40 for |c_bg| <= 256 (a larger
+// background keeps the updates, and so does the aux output, which returns T).
+// The frozen value stays an upper bound of T.
 #include "mgs_internal.cuh"
 
 namespace mgs {
 namespace {
 
-constexpr int kThreads = 64;
+constexpr int kThreads = 128;
 constexpr int kWarps = kThreads / 32;
+constexpr float kFrozenT = 0.000244140625f;   // 2^-12
+constexpr float kMaxFrozenBg = 256.0f;
+constexpr int kFreezeEvery = 128;             // list entries between two checks
+constexpr float kLogClamp = -0.014499569695115089f;   // log2(0.99)
 
 typedef unsigned long long f2;  // two packed FP32 lanes
 
@@ -58,95 +72,202 @@ __device__ __forceinline__ float ex2(float x) {
     return y;
 }
 
-// Staged Gaussian: five 16-byte words of duplicated pairs, so every operand
-// of the packed arithmetic comes straight from one shared-memory load.
+// Staged Gaussian of the FMA sums: five 16-byte words of duplicated pairs, so
+// every operand of the packed arithmetic comes straight from one shared-memory
+// load.
 //   s0 = {m_x, m_x, m_y, m_y}      s1 = {l11, l11, l21, l21}
 //   s2 = {l22, l22, log2 o, log2 o} s3 = {-w, -w, -w c_r, -w c_r}
-//   s4 = {-w c_g, -w c_g, -w c_b, -w c_b}
+//   s4 = {-w c_g, -w c_g, -w c_b, -w c_b}, depth image: s5 = {-w d, -w d, 0, 0}
+constexpr int kGroup = 4;         // candidates per step: one per lane of a quad
+constexpr int kRingF = 36;        // slots per warp: 32 + 3 left over, whole groups
+template <bool kDepth>
+struct FmaSmem {
+    ulonglong2 s[kWarps][kDepth ? 6 : 5][kRingF];
+};
 
-// Accumulates one staged Gaussian into a thread's four pixels (two pairs).
-template <bool kCount, bool kDepth>
-__device__ __forceinline__ void accumulate(const ulonglong2 (*wb)[32], int k, f2 pxa, f2 pxb,
-                                           f2 pyc, f2 kq2, f2 (&A)[2][3], f2 (&B)[2],
-                                           f2 (&T)[2], f2 (&AD)[2], int (&cnt)[4]) {
+// The sums of one lane: its row's eight pixels as four pairs.
+template <bool kDepth>
+struct FmaSums {
+    f2 A[4][3], B[4], T[4], AD[kDepth ? 4 : 1];
+};
+
+// Accumulates one staged Gaussian (slot k of the warp's ring) into the lane's
+// eight pixels.  kClamp: its opacity may exceed 0.99; kLive: T is updated.
+template <bool kCount, bool kDepth, bool kClamp, bool kLive>
+__device__ __forceinline__ void accumulate(const ulonglong2 (*wb)[kRingF], int k, const f2 (&px)[4],
+                                           f2 pyc, f2 kq2, FmaSums<kDepth> &S, int (&cnt)[8]) {
     const ulonglong2 s0 = wb[0][k], s1 = wb[1][k], s2 = wb[2][k];
-    // inclusion test (exact FP32 sequence); the row terms are shared by both pairs
+    // inclusion test (exact FP32 sequence); the row terms are shared by the pairs
     const f2 dy = sub2(pyc, s0.y);
     const f2 ldy = mul2(s1.y, dy);
     const f2 e2 = mul2(s2.x, dy);
     const f2 e2s = mul2(e2, e2);
-    const f2 dxa = sub2(pxa, s0.x);
-    const f2 dxb = sub2(pxb, s0.x);
-    const f2 e1a = fma2(s1.x, dxa, ldy);
-    const f2 e1b = fma2(s1.x, dxb, ldy);
-    const f2 qa = fma2(e1a, e1a, e2s);
-    const f2 qb = fma2(e1b, e1b, e2s);
-    // a = min(0.99, o 2^(-q log2(e) / 2)), kept negated
-    const f2 ga = fma2(qa, kq2, s2.y);
-    const f2 gb = fma2(qb, kq2, s2.y);
-    float q[4], g[4], n[4];
-    upk(qa, q[0], q[1]);
-    upk(qb, q[2], q[3]);
-    upk(ga, g[0], g[1]);
-    upk(gb, g[2], g[3]);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        n[i] = q[i] <= 9.0f ? fmaxf(-ex2(g[i]), -0.99f) : 0.0f;
-        if (kCount) cnt[i] += q[i] <= 9.0f;
-    }
     const ulonglong2 s3 = wb[3][k], s4 = wb[4][k];
-    const f2 na[2] = {pk(n[0], n[1]), pk(n[2], n[3])};
+    f2 wd = 0ull;
+    if constexpr (kDepth) wd = wb[5][k].x;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        A[h][0] = fma2(na[h], s3.y, A[h][0]);
-        A[h][1] = fma2(na[h], s4.x, A[h][1]);
-        A[h][2] = fma2(na[h], s4.y, A[h][2]);
-        B[h] = fma2(na[h], s3.x, B[h]);
-        T[h] = fma2(na[h], T[h], T[h]);
-    }
-    if (kDepth) {
-        const ulonglong2 s5 = wb[5][k];   // {-w d, -w d, 0, 0}
-        AD[0] = fma2(na[0], s5.x, AD[0]);
-        AD[1] = fma2(na[1], s5.x, AD[1]);
+    for (int p = 0; p < 4; ++p) {
+        const f2 e1 = fma2(s1.x, sub2(px[p], s0.x), ldy);
+        const f2 q = fma2(e1, e1, e2s);
+        // a = min(0.99, o 2^(-q log2(e) / 2)), kept negated
+        const f2 g = fma2(q, kq2, s2.y);
+        float q0, q1, g0, g1;
+        upk(q, q0, q1);
+        upk(g, g0, g1);
+        float n0 = -ex2(g0), n1 = -ex2(g1);
+        if constexpr (kClamp) {
+            n0 = fmaxf(n0, -0.99f);
+            n1 = fmaxf(n1, -0.99f);
+        }
+        n0 = q0 <= 9.0f ? n0 : 0.0f;
+        n1 = q1 <= 9.0f ? n1 : 0.0f;
+        if constexpr (kCount) {
+            cnt[2 * p] += q0 <= 9.0f;
+            cnt[2 * p + 1] += q1 <= 9.0f;
+        }
+        const f2 na = pk(n0, n1);
+        S.A[p][0] = fma2(na, s3.y, S.A[p][0]);
+        S.A[p][1] = fma2(na, s4.x, S.A[p][1]);
+        S.A[p][2] = fma2(na, s4.y, S.A[p][2]);
+        S.B[p] = fma2(na, s3.x, S.B[p]);
+        if constexpr (kLive) S.T[p] = fma2(na, S.T[p], S.T[p]);
+        if constexpr (kDepth) S.AD[p] = fma2(na, wd, S.AD[p]);
     }
 }
 
-// Rasterises one tile with one CTA (two warps); warp w owns the 16x8 pixel
-// block of rows 8w..8w+7, lane l the four pixels (4 (l & 3) .. +3, l >> 2) of
-// that block.  Each warp streams the tile's list on its own (no block-wide
-// barrier): 32 entries at a time, one per lane (the next 32 are fetched while
-// the current ones are accumulated), are tested against the warp's block,
-// compacted into the warp's shared-memory buffer (ballot) and accumulated by
-// all lanes.
+// Does every lane hold partial products of at most kFrozenT?
+__device__ __forceinline__ bool all_frozen(float m) {
+    return __all_sync(0xffffffffu, m <= kFrozenT);
+}
+
+__device__ __forceinline__ bool may_freeze(const RenderArgs &args) {
+    return fmaxf(fmaxf(fabsf(args.bg[0]), fabsf(args.bg[1])), fabsf(args.bg[2])) <= kMaxFrozenBg;
+}
+
+// Writes one pixel's outputs from its sums.
+template <bool kAux, bool kCount, bool kDepth>
+__device__ __forceinline__ void put_pixel(const RenderArgs &args, int x, int y, float ar, float ag,
+                                          float ab, float bb, float tr, int cnt, float ad) {
+    const DevCamera &cam = args.cam;
+    const int64_t HW = (int64_t)cam.width * cam.height;
+    const int64_t p = (int64_t)y * cam.width + x;
+    const float fg = bb > 0.0f ? (1.0f - tr) / bb : 0.0f;
+    float *out = args.out_rgb + 3 * p;
+    out[0] = fmaf(fg, ar, tr * args.bg[0]);
+    out[1] = fmaf(fg, ag, tr * args.bg[1]);
+    out[2] = fmaf(fg, ab, tr * args.bg[2]);
+    if (kAux) {
+        args.out_aux[p] = ar;
+        args.out_aux[HW + p] = ag;
+        args.out_aux[2 * HW + p] = ab;
+        args.out_aux[3 * HW + p] = bb;
+        args.out_aux[4 * HW + p] = tr;
+    }
+    if (kCount) args.out_count[p] = cnt;
+    if (kDepth) args.out_depth[p] = bb > 0.0f ? ad / bb : 0.0f;
+}
+
+// Sum over the quad of a lane's four pixel pairs: lane t of the quad receives
+// pair t (reduce-scatter: half of the pairs to the other half of the quad,
+// then one to the neighbour).
+__device__ __forceinline__ float2 quad_sum(const f2 (&v)[4], int t) {
+    float x[4][2];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) upk(v[p], x[p][0], x[p][1]);
+    float y[2][2];
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float send = (t & 2) ? x[p][h] : x[p + 2][h];
+            y[p][h] = ((t & 2) ? x[p + 2][h] : x[p][h]) + __shfl_xor_sync(0xffffffffu, send, 2);
+        }
+    float z[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const float send = (t & 1) ? y[0][h] : y[1][h];
+        z[h] = ((t & 1) ? y[1][h] : y[0][h]) + __shfl_xor_sync(0xffffffffu, send, 1);
+    }
+    return make_float2(z[0], z[1]);
+}
+// The same with products (T).
+__device__ __forceinline__ float2 quad_product(const f2 (&v)[4], int t) {
+    float2 r = make_float2(1.0f, 1.0f);
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        float x, y;
+        upk(v[p], x, y);
+        x *= __shfl_xor_sync(0xffffffffu, x, 1);
+        y *= __shfl_xor_sync(0xffffffffu, y, 1);
+        x *= __shfl_xor_sync(0xffffffffu, x, 2);
+        y *= __shfl_xor_sync(0xffffffffu, y, 2);
+        if (p == t) r = make_float2(x, y);
+    }
+    return r;
+}
+
+// Rasterises one tile on the FMA pipe (four warps).  Each warp streams the
+// tile's list on its own (no block-wide barrier): 32 entries at a time, one per
+// lane (list entries are fetched two batches ahead, their records one batch
+// ahead), are tested against the warp's block and queued in its ring; groups
+// of four candidates are accumulated, one per lane of each quad.
+//
+// Bound: issue (36 packed operations and about 69 instructions per lane,
+// candidate and eight pixels).  With two warps of 16x8 pixels per tile and four
+// pixels per lane, every candidate's operands and row terms served four pixels
+// instead of eight, 14 % more (block, Gaussian) pairs were evaluated, and small
+// images had half the warps: 0.212 ms at 160k Gaussians, 1001x667, against
+// 0.167 ms; 29 against 20 us at 4k, 256x256; 0.51 against 0.46 ms for the
+// training forward (300k, 1296x840).
 template <bool kAux, bool kCount, bool kDepth = false>
-__device__ __forceinline__ void raster_tile(const RenderArgs &args, int tile,
-                                            ulonglong2 (*buf)[kDepth ? 6 : 5][32]) {
+__device__ __forceinline__ void raster_tile(const RenderArgs &args, int tile, FmaSmem<kDepth> &sm) {
     const DevCamera &cam = args.cam;
     const int tx = tile % cam.tiles_x, ty = tile / cam.tiles_x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int bx0 = tx * kTile, by0 = ty * kTile + 8 * warp;
-    const int px = bx0 + 4 * (lane & 3);
-    const int py = by0 + (lane >> 2);
+    const int g = lane >> 2, t = lane & 3;
+    const int bx0 = tx * kTile + 8 * (warp & 1), by0 = ty * kTile + 8 * (warp >> 1);
+    const int py = by0 + g;
 
     const uint32_t start = args.tile_offsets[tile];
     const uint32_t end = args.tile_offsets[tile + 1];
     const bool no_cull = (args.flags & MGS_FLAG_NO_CULL) != 0;
-    const float bx = (float)bx0 + 8.0f, by = (float)by0 + 4.0f;
+    const float bcx = (float)bx0 + 4.0f, bcy = (float)by0 + 4.0f;
 
-    const f2 pxa = pk((float)px + 0.5f, (float)px + 1.5f);
-    const f2 pxb = pk((float)px + 2.5f, (float)px + 3.5f);
+    f2 px[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) px[p] = pk((float)(bx0 + 2 * p) + 0.5f, (float)(bx0 + 2 * p) + 1.5f);
     const f2 pyc = pk((float)py + 0.5f, (float)py + 0.5f);
     const float kq = -0.72134752044448170f;  // -log2(e) / 2
     const f2 kq2 = pk(kq, kq);
-    f2 A[2][3] = {{0ull, 0ull, 0ull}, {0ull, 0ull, 0ull}};
-    f2 B[2] = {0ull, 0ull};
-    f2 T[2] = {pk(1.0f, 1.0f), pk(1.0f, 1.0f)};
-    f2 AD[2] = {0ull, 0ull};
-    int cnt[4] = {0, 0, 0, 0};
-    ulonglong2(*wb)[32] = buf[warp];
+    FmaSums<kDepth> S;
+    int cnt[8];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        S.A[p][0] = S.A[p][1] = S.A[p][2] = S.B[p] = 0ull;
+        S.T[p] = pk(1.0f, 1.0f);
+        if constexpr (kDepth) S.AD[p] = 0ull;
+        cnt[2 * p] = cnt[2 * p + 1] = 0;
+    }
+    ulonglong2(*wb)[kRingF] = sm.s[warp];
 
-    // list entries two batches ahead, their records one batch ahead (the
-    // dependent record loads never wait on the list load)
+    int head = 0, count = 0;   // queued candidates: ring slots [head, head + count) mod kRingF
+    int clamp_left = 0;        // queued candidates up to the last whose opacity exceeds 0.99
+    bool live = true;          // T is still updated
+    const bool freeze = !kAux && may_freeze(args);
+    auto group = [&]() {
+        const int k = head + t;
+        if (live) {
+            if (clamp_left > 0) accumulate<kCount, kDepth, true, true>(wb, k, px, pyc, kq2, S, cnt);
+            else accumulate<kCount, kDepth, false, true>(wb, k, px, pyc, kq2, S, cnt);
+        } else if constexpr (!kAux) {
+            if (clamp_left > 0) accumulate<kCount, kDepth, true, false>(wb, k, px, pyc, kq2, S, cnt);
+            else accumulate<kCount, kDepth, false, false>(wb, k, px, pyc, kq2, S, cnt);
+        }
+        clamp_left -= kGroup;
+        count -= kGroup;
+        head += kGroup;
+        if (head == kRingF) head = 0;
+    };
     float4 a_n = make_float4(0.f, 0.f, 0.f, 0.f), b_n = a_n, c_n = a_n;
     uint32_t gid_nn = 0;
     if (start + lane < end) {
@@ -160,7 +281,7 @@ __device__ __forceinline__ void raster_tile(const RenderArgs &args, int tile,
         const uint32_t j = base + lane;
         const float4 a = a_n, b = b_n, c = c_n;
         const bool cand =
-            j < end && (no_cull || block_may_hit(a.x, a.y, a.z, a.w, b.x, bx, by, 7.5f, 3.5f));
+            j < end && (no_cull || block_may_hit(a.x, a.y, a.z, a.w, b.x, bcx, bcy, 3.5f, 3.5f));
         if (j + 32 < end) {
             const uint32_t gid = gid_nn;
             a_n = __ldg(&args.rec[gid].a);
@@ -169,55 +290,71 @@ __device__ __forceinline__ void raster_tile(const RenderArgs &args, int tile,
         }
         if (j + 64 < end) gid_nn = __ldg(&args.gids[j + 64]);
         const unsigned bal = __ballot_sync(0xffffffffu, cand);
+        const unsigned cb = __ballot_sync(0xffffffffu, cand && !(b.y <= kLogClamp));
         if (cand) {
-            const int pos = __popc(bal & ((1u << lane) - 1u));
+            int pos = head + count + __popc(bal & ((1u << lane) - 1u));
+            if (pos >= kRingF) pos -= kRingF;
             wb[0][pos] = make_ulonglong2(pk(a.x, a.x), pk(a.y, a.y));
             wb[1][pos] = make_ulonglong2(pk(a.z, a.z), pk(a.w, a.w));
             wb[2][pos] = make_ulonglong2(pk(b.x, b.x), pk(b.y, b.y));
             wb[3][pos] = make_ulonglong2(pk(b.z, b.z), pk(b.w, b.w));
             wb[4][pos] = make_ulonglong2(pk(c.x, c.x), pk(c.y, c.y));
-            if (kDepth) wb[5][pos] = make_ulonglong2(pk(c.w, c.w), 0ull);   // -w d
+            if constexpr (kDepth) wb[5][pos] = make_ulonglong2(pk(c.w, c.w), 0ull);   // -w d
+        }
+        if (cb) clamp_left = count + __popc(bal & (0xffffffffu >> __clz(cb)));
+        __syncwarp();
+        count += __popc(bal);
+        while (count >= kGroup) group();
+        if (freeze && live && ((base - start) & (kFreezeEvery - 1)) == kFreezeEvery - 32) {
+            float m = 0.0f;
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                float x, y;
+                upk(S.T[p], x, y);
+                m = fmaxf(m, fmaxf(x, y));
+                if (!(x <= 1.0f && y <= 1.0f)) m = 1.0f;   // NaN: keep updating
+            }
+            live = !all_frozen(m);
         }
         __syncwarp();
-        const int nc = __popc(bal);
-#pragma unroll 2
-        for (int k = 0; k < nc; ++k)
-            accumulate<kCount, kDepth>(wb, k, pxa, pxb, pyc, kq2, A, B, T, AD, cnt);
+    }
+    if (count > 0) {   // pad the last group with entries that include no pixel and weigh 0
+        if (lane < kGroup - count) {
+            int pos = head + count + lane;
+            if (pos >= kRingF) pos -= kRingF;
+            wb[0][pos] = make_ulonglong2(pk(1e30f, 1e30f), pk(1e30f, 1e30f));
+            wb[1][pos] = make_ulonglong2(pk(1.0f, 1.0f), 0ull);
+            wb[2][pos] = make_ulonglong2(pk(1.0f, 1.0f), 0ull);
+            wb[3][pos] = wb[4][pos] = make_ulonglong2(0ull, 0ull);
+            if constexpr (kDepth) wb[5][pos] = make_ulonglong2(0ull, 0ull);
+        }
         __syncwarp();
+        group();
     }
 
-    if (py >= cam.height) return;
-    float ar[4], ag[4], ab[4], bb[4], tt[4], ad[4];
+    // lane t of a quad receives the sums of pixels 2t, 2t + 1
+    const f2 Ar[4] = {S.A[0][0], S.A[1][0], S.A[2][0], S.A[3][0]};
+    const f2 Ag[4] = {S.A[0][1], S.A[1][1], S.A[2][1], S.A[3][1]};
+    const f2 Ab[4] = {S.A[0][2], S.A[1][2], S.A[2][2], S.A[3][2]};
+    const float2 ar = quad_sum(Ar, t), ag = quad_sum(Ag, t), ab = quad_sum(Ab, t);
+    const float2 bb = quad_sum(S.B, t), tr = quad_product(S.T, t);
+    float2 ad = make_float2(0.f, 0.f);
+    if constexpr (kDepth) ad = quad_sum(S.AD, t);
+    int c2[2] = {0, 0};
+    if constexpr (kCount) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        upk(AD[h], ad[2 * h], ad[2 * h + 1]);
-        upk(A[h][0], ar[2 * h], ar[2 * h + 1]);
-        upk(A[h][1], ag[2 * h], ag[2 * h + 1]);
-        upk(A[h][2], ab[2 * h], ab[2 * h + 1]);
-        upk(B[h], bb[2 * h], bb[2 * h + 1]);
-        upk(T[h], tt[2 * h], tt[2 * h + 1]);
-    }
-    const int64_t HW = (int64_t)cam.width * cam.height;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int x = px + k;
-        if (x >= cam.width) break;
-        const int64_t p = (int64_t)py * cam.width + x;
-        const float fg = bb[k] > 0.0f ? (1.0f - tt[k]) / bb[k] : 0.0f;
-        float *o = args.out_rgb + 3 * p;
-        o[0] = fmaf(fg, ar[k], tt[k] * args.bg[0]);
-        o[1] = fmaf(fg, ag[k], tt[k] * args.bg[1]);
-        o[2] = fmaf(fg, ab[k], tt[k] * args.bg[2]);
-        if (kAux) {
-            args.out_aux[p] = ar[k];
-            args.out_aux[HW + p] = ag[k];
-            args.out_aux[2 * HW + p] = ab[k];
-            args.out_aux[3 * HW + p] = bb[k];
-            args.out_aux[4 * HW + p] = tt[k];
+        for (int k = 0; k < 8; ++k) {
+            int x = cnt[k];
+            x += __shfl_xor_sync(0xffffffffu, x, 1);
+            x += __shfl_xor_sync(0xffffffffu, x, 2);
+            if ((k >> 1) == t) c2[k & 1] = x;
         }
-        if (kCount) args.out_count[p] = cnt[k];
-        if (kDepth) args.out_depth[p] = bb[k] > 0.0f ? ad[k] / bb[k] : 0.0f;
     }
+    const int x = bx0 + 2 * t;
+    if (py >= cam.height || x >= cam.width) return;
+    put_pixel<kAux, kCount, kDepth>(args, x, py, ar.x, ag.x, ab.x, bb.x, tr.x, c2[0], ad.x);
+    if (x + 1 < cam.width)
+        put_pixel<kAux, kCount, kDepth>(args, x + 1, py, ar.y, ag.y, ab.y, bb.y, tr.y, c2[1], ad.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -238,8 +375,6 @@ __device__ __forceinline__ void raster_tile(const RenderArgs &args, int tile,
 // when the frame's largest weight would overflow FP16 (the scale cancels in
 // A / B and is divided out here).  T stays in FP32 FMAs.  Tiles listing a Gaussian
 // outside that scale's range (kTileWide) are rasterised by the FMA tile code.
-constexpr int kTcThreads = 128;
-constexpr int kTcWarps = kTcThreads / 32;
 constexpr int kChunk = 8;        // candidates per MMA (K)
 constexpr int kRing = 64;        // candidate slots per warp: eight chunks (a power of two)
 
@@ -249,9 +384,9 @@ constexpr int kRing = 64;        // candidate slots per warp: eight chunks (a po
 //   geo[1][s / 2] = {l11(a), l11(b), l21(a), l21(b)}
 //   geo[2][s / 2] = {l22(a), l22(b), log2 o(a), log2 o(b)}   (a = even slot)
 struct TcSmem {
-    float4 geo[kTcWarps][3][kRing / 2];
-    uint4 wt[kTcWarps][kRing];            // slot s: its 8 FP16 weight columns
-    float2 wd[kTcWarps][kRing / 2];       // depth image only: w d of slots 2p, 2p + 1
+    float4 geo[kWarps][3][kRing / 2];
+    uint4 wt[kWarps][kRing];            // slot s: its 8 FP16 weight columns
+    float2 wd[kWarps][kRing / 2];       // depth image only: w d of slots 2p, 2p + 1
 };
 
 __device__ __forceinline__ uint32_t h2bits(float lo, float hi) {
@@ -337,7 +472,6 @@ __device__ __forceinline__ void raster_tile_tc(const RenderArgs &args, int tile,
     // weight scale 2^(14 - e) when the frame's largest weight has exponent e >= 14
     const int we = (int)((args.status->wmax_frame_bits >> 23) & 0xFFu) - 127;
     const float wscale = we >= 14 ? __int_as_float((127 + 14 - we) << 23) : 1.0f;
-    const float kLogClamp = -0.014499569695115089f;   // log2(0.99)
 
     f2 pxc[8];
 #pragma unroll
@@ -523,6 +657,162 @@ __device__ __forceinline__ void raster_tile_tc(const RenderArgs &args, int tile,
     }
 }
 
+// Accumulates one staged Gaussian into a thread's four pixels (two pairs).
+template <bool kCount, bool kDepth>
+__device__ __forceinline__ void accumulate_wide(const ulonglong2 (*wb)[32], int k, f2 pxa, f2 pxb,
+                                           f2 pyc, f2 kq2, f2 (&A)[2][3], f2 (&B)[2],
+                                           f2 (&T)[2], f2 (&AD)[2], int (&cnt)[4]) {
+    const ulonglong2 s0 = wb[0][k], s1 = wb[1][k], s2 = wb[2][k];
+    // inclusion test (exact FP32 sequence); the row terms are shared by both pairs
+    const f2 dy = sub2(pyc, s0.y);
+    const f2 ldy = mul2(s1.y, dy);
+    const f2 e2 = mul2(s2.x, dy);
+    const f2 e2s = mul2(e2, e2);
+    const f2 dxa = sub2(pxa, s0.x);
+    const f2 dxb = sub2(pxb, s0.x);
+    const f2 e1a = fma2(s1.x, dxa, ldy);
+    const f2 e1b = fma2(s1.x, dxb, ldy);
+    const f2 qa = fma2(e1a, e1a, e2s);
+    const f2 qb = fma2(e1b, e1b, e2s);
+    // a = min(0.99, o 2^(-q log2(e) / 2)), kept negated
+    const f2 ga = fma2(qa, kq2, s2.y);
+    const f2 gb = fma2(qb, kq2, s2.y);
+    float q[4], g[4], n[4];
+    upk(qa, q[0], q[1]);
+    upk(qb, q[2], q[3]);
+    upk(ga, g[0], g[1]);
+    upk(gb, g[2], g[3]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        n[i] = q[i] <= 9.0f ? fmaxf(-ex2(g[i]), -0.99f) : 0.0f;
+        if (kCount) cnt[i] += q[i] <= 9.0f;
+    }
+    const ulonglong2 s3 = wb[3][k], s4 = wb[4][k];
+    const f2 na[2] = {pk(n[0], n[1]), pk(n[2], n[3])};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        A[h][0] = fma2(na[h], s3.y, A[h][0]);
+        A[h][1] = fma2(na[h], s4.x, A[h][1]);
+        A[h][2] = fma2(na[h], s4.y, A[h][2]);
+        B[h] = fma2(na[h], s3.x, B[h]);
+        T[h] = fma2(na[h], T[h], T[h]);
+    }
+    if (kDepth) {
+        const ulonglong2 s5 = wb[5][k];   // {-w d, -w d, 0, 0}
+        AD[0] = fma2(na[0], s5.x, AD[0]);
+        AD[1] = fma2(na[1], s5.x, AD[1]);
+    }
+}
+
+// FMA tile code of wide tiles in the tensor-core kernels (two warps); warp w owns the 16x8 pixel
+// block of rows 8w..8w+7, lane l the four pixels (4 (l & 3) .. +3, l >> 2) of
+// that block.  Each warp streams the tile's list on its own (no block-wide
+// barrier): 32 entries at a time, one per lane (the next 32 are fetched while
+// the current ones are accumulated), are tested against the warp's block,
+// compacted into the warp's shared-memory buffer (ballot) and accumulated by
+// all lanes.
+template <bool kAux, bool kCount, bool kDepth = false>
+__device__ __forceinline__ void raster_tile_wide(const RenderArgs &args, int tile,
+                                            ulonglong2 (*buf)[kDepth ? 6 : 5][32]) {
+    const DevCamera &cam = args.cam;
+    const int tx = tile % cam.tiles_x, ty = tile / cam.tiles_x;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int bx0 = tx * kTile, by0 = ty * kTile + 8 * warp;
+    const int px = bx0 + 4 * (lane & 3);
+    const int py = by0 + (lane >> 2);
+
+    const uint32_t start = args.tile_offsets[tile];
+    const uint32_t end = args.tile_offsets[tile + 1];
+    const bool no_cull = (args.flags & MGS_FLAG_NO_CULL) != 0;
+    const float bx = (float)bx0 + 8.0f, by = (float)by0 + 4.0f;
+
+    const f2 pxa = pk((float)px + 0.5f, (float)px + 1.5f);
+    const f2 pxb = pk((float)px + 2.5f, (float)px + 3.5f);
+    const f2 pyc = pk((float)py + 0.5f, (float)py + 0.5f);
+    const float kq = -0.72134752044448170f;  // -log2(e) / 2
+    const f2 kq2 = pk(kq, kq);
+    f2 A[2][3] = {{0ull, 0ull, 0ull}, {0ull, 0ull, 0ull}};
+    f2 B[2] = {0ull, 0ull};
+    f2 T[2] = {pk(1.0f, 1.0f), pk(1.0f, 1.0f)};
+    f2 AD[2] = {0ull, 0ull};
+    int cnt[4] = {0, 0, 0, 0};
+    ulonglong2(*wb)[32] = buf[warp];
+
+    // list entries two batches ahead, their records one batch ahead (the
+    // dependent record loads never wait on the list load)
+    float4 a_n = make_float4(0.f, 0.f, 0.f, 0.f), b_n = a_n, c_n = a_n;
+    uint32_t gid_nn = 0;
+    if (start + lane < end) {
+        const uint32_t gid = __ldg(&args.gids[start + lane]);
+        a_n = __ldg(&args.rec[gid].a);
+        b_n = __ldg(&args.rec[gid].b);
+        c_n = __ldg(&args.rec[gid].c);
+    }
+    if (start + 32 + lane < end) gid_nn = __ldg(&args.gids[start + 32 + lane]);
+    for (uint32_t base = start; base < end; base += 32) {
+        const uint32_t j = base + lane;
+        const float4 a = a_n, b = b_n, c = c_n;
+        const bool cand =
+            j < end && (no_cull || block_may_hit(a.x, a.y, a.z, a.w, b.x, bx, by, 7.5f, 3.5f));
+        if (j + 32 < end) {
+            const uint32_t gid = gid_nn;
+            a_n = __ldg(&args.rec[gid].a);
+            b_n = __ldg(&args.rec[gid].b);
+            c_n = __ldg(&args.rec[gid].c);
+        }
+        if (j + 64 < end) gid_nn = __ldg(&args.gids[j + 64]);
+        const unsigned bal = __ballot_sync(0xffffffffu, cand);
+        if (cand) {
+            const int pos = __popc(bal & ((1u << lane) - 1u));
+            wb[0][pos] = make_ulonglong2(pk(a.x, a.x), pk(a.y, a.y));
+            wb[1][pos] = make_ulonglong2(pk(a.z, a.z), pk(a.w, a.w));
+            wb[2][pos] = make_ulonglong2(pk(b.x, b.x), pk(b.y, b.y));
+            wb[3][pos] = make_ulonglong2(pk(b.z, b.z), pk(b.w, b.w));
+            wb[4][pos] = make_ulonglong2(pk(c.x, c.x), pk(c.y, c.y));
+            if (kDepth) wb[5][pos] = make_ulonglong2(pk(c.w, c.w), 0ull);   // -w d
+        }
+        __syncwarp();
+        const int nc = __popc(bal);
+#pragma unroll 2
+        for (int k = 0; k < nc; ++k)
+            accumulate_wide<kCount, kDepth>(wb, k, pxa, pxb, pyc, kq2, A, B, T, AD, cnt);
+        __syncwarp();
+    }
+
+    if (py >= cam.height) return;
+    float ar[4], ag[4], ab[4], bb[4], tt[4], ad[4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        upk(AD[h], ad[2 * h], ad[2 * h + 1]);
+        upk(A[h][0], ar[2 * h], ar[2 * h + 1]);
+        upk(A[h][1], ag[2 * h], ag[2 * h + 1]);
+        upk(A[h][2], ab[2 * h], ab[2 * h + 1]);
+        upk(B[h], bb[2 * h], bb[2 * h + 1]);
+        upk(T[h], tt[2 * h], tt[2 * h + 1]);
+    }
+    const int64_t HW = (int64_t)cam.width * cam.height;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int x = px + k;
+        if (x >= cam.width) break;
+        const int64_t p = (int64_t)py * cam.width + x;
+        const float fg = bb[k] > 0.0f ? (1.0f - tt[k]) / bb[k] : 0.0f;
+        float *o = args.out_rgb + 3 * p;
+        o[0] = fmaf(fg, ar[k], tt[k] * args.bg[0]);
+        o[1] = fmaf(fg, ag[k], tt[k] * args.bg[1]);
+        o[2] = fmaf(fg, ab[k], tt[k] * args.bg[2]);
+        if (kAux) {
+            args.out_aux[p] = ar[k];
+            args.out_aux[HW + p] = ag[k];
+            args.out_aux[2 * HW + p] = ab[k];
+            args.out_aux[3 * HW + p] = bb[k];
+            args.out_aux[4 * HW + p] = tt[k];
+        }
+        if (kCount) args.out_count[p] = cnt[k];
+        if (kDepth) args.out_depth[p] = bb[k] > 0.0f ? ad[k] / bb[k] : 0.0f;
+    }
+}
+
 // Tensor-core accumulation is used for FP16-attribute scenes unless the
 // caller asks for the FP32 FMA sums.
 __host__ __device__ __forceinline__ bool use_tc(const RenderArgs &a) { return tc_raster(a); }
@@ -530,25 +820,24 @@ __host__ __device__ __forceinline__ bool use_tc(const RenderArgs &a) { return tc
 // One CTA per tile, longest tile lists first.
 template <bool kAux, bool kCount, bool kDepth = false>
 __global__ void __launch_bounds__(kThreads) k_raster(RenderArgs args) {
-    __shared__ ulonglong2 buf[kWarps][kDepth ? 6 : 5][32];
+    __shared__ FmaSmem<kDepth> sm;
     if (args.status->last_pairs > args.capacity) return;  // overflowed: lists incomplete
-    raster_tile<kAux, kCount, kDepth>(args, (int)(args.tile_order[blockIdx.x] & kTileMask), buf);
+    raster_tile<kAux, kCount, kDepth>(args, (int)(args.tile_order[blockIdx.x] & kTileMask), sm);
 }
 
 // Tiles that list a Gaussian whose weight the FP16 sums cannot hold next to
-// the others (kTileWide, see kWideWeight) take the FP32 FMA tile code on the
-// CTA's first two warps.
+// the others (kTileWide, see kWideWeight) take the FP32 FMA tile code.
 template <bool kAux, bool kCount, bool kDepth = false>
-__global__ void __launch_bounds__(kTcThreads) k_raster_tc(RenderArgs args) {
+__global__ void __launch_bounds__(kThreads) k_raster_tc(RenderArgs args) {
     __shared__ union {
         TcSmem tc;
-        ulonglong2 buf[kWarps][kDepth ? 6 : 5][32];
+        ulonglong2 buf[2][kDepth ? 6 : 5][32];
     } sm;
     if (args.status->last_pairs > args.capacity) return;  // overflowed: lists incomplete
     const uint32_t ord = args.tile_order[blockIdx.x];
     const int tile = (int)(ord & kTileMask);
     if (ord & kTileWide) {
-        if (threadIdx.x < kThreads) raster_tile<kAux, kCount, kDepth>(args, tile, sm.buf);
+        if (threadIdx.x < 64) raster_tile_wide<kAux, kCount, kDepth>(args, tile, sm.buf);
     } else {
         raster_tile_tc<kAux, kCount, kDepth>(args, tile, sm.tc);
     }
@@ -558,14 +847,14 @@ __global__ void __launch_bounds__(kTcThreads) k_raster_tc(RenderArgs args) {
 // resolutions) form one work list; resident CTAs pull (view, tile) items from
 // an atomic counter until the list is exhausted.  Items are numbered view by
 // view (prefix[v] = first item of view v), each view's tiles longest first.
-// A CTA has four warps: FP16 views use all four (tensor-core sums), FP32
-// views and wide tiles (kTileWide) the first two (FMA sums).
-__global__ void __launch_bounds__(kTcThreads) k_raster_batch(const RenderArgs *__restrict__ views,
+// FP16 views use all four warps (tensor-core sums), FP32 views and wide tiles
+// (kTileWide) the first two (FMA sums).
+__global__ void __launch_bounds__(kThreads) k_raster_batch(const RenderArgs *__restrict__ views,
                                                              const int *__restrict__ prefix,
                                                              int nviews,
                                                              unsigned *__restrict__ counter) {
     __shared__ union {
-        ulonglong2 buf[kWarps][5][32];
+        ulonglong2 buf[2][5][32];
         TcSmem tc;
     } sm;
     __shared__ int item_s;
@@ -587,8 +876,8 @@ __global__ void __launch_bounds__(kTcThreads) k_raster_batch(const RenderArgs *_
         const int tile = (int)(ord & kTileMask);
         if (use_tc(a) && !(ord & kTileWide))
             raster_tile_tc<false, false>(a, tile, sm.tc);
-        else if (threadIdx.x < kThreads)
-            raster_tile<false, false>(a, tile, sm.buf);
+        else if (threadIdx.x < 64)
+            raster_tile_wide<false, false>(a, tile, sm.buf);
     }
 }
 
@@ -596,7 +885,7 @@ template <bool kAux, bool kCount>
 cudaError_t launch_t(const RenderArgs &a, cudaStream_t stream) {
     const int T = a.cam.tiles_x * a.cam.tiles_y;
     if (use_tc(a))
-        k_raster_tc<kAux, kCount><<<T, kTcThreads, 0, stream>>>(a);
+        k_raster_tc<kAux, kCount><<<T, kThreads, 0, stream>>>(a);
     else
         k_raster<kAux, kCount><<<T, kThreads, 0, stream>>>(a);
     return cudaGetLastError();
@@ -608,7 +897,7 @@ cudaError_t launch_raster(const RenderArgs &a, cudaStream_t stream) {
     const bool aux = a.out_aux != nullptr, cnt = a.out_count != nullptr;
     if (a.out_depth) {   // depth image (Eq. 5), no aux / count outputs
         if (use_tc(a))
-            k_raster_tc<false, false, true><<<a.cam.tiles_x * a.cam.tiles_y, kTcThreads, 0, stream>>>(a);
+            k_raster_tc<false, false, true><<<a.cam.tiles_x * a.cam.tiles_y, kThreads, 0, stream>>>(a);
         else
             k_raster<false, false, true><<<a.cam.tiles_x * a.cam.tiles_y, kThreads, 0, stream>>>(a);
         return cudaGetLastError();
@@ -628,10 +917,10 @@ cudaError_t launch_raster_batch(const RenderArgs *views_dev, const int *prefix_d
     cudaError_t e = cudaMemsetAsync(counter_dev, 0, sizeof(unsigned), stream);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_raster_batch, kTcThreads, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_raster_batch, kThreads, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    k_raster_batch<<<sm_count * per_sm, kTcThreads, 0, stream>>>(views_dev, prefix_dev, nviews,
+    k_raster_batch<<<sm_count * per_sm, kThreads, 0, stream>>>(views_dev, prefix_dev, nviews,
                                                                  counter_dev);
     return cudaGetLastError();
 }
