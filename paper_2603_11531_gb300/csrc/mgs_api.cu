@@ -283,6 +283,7 @@ mgs_status render_impl(mgs_workspace w, mgs_scene s, const mgs_camera *cam,
     a.perm = s->perm;
     a.iperm = s->iperm;
     a.tile_count = w->tile_count;
+    a.group_cost = bin_group_cost(w->bases, s->n, T, w->ctx->sm_count);
     a.tile_offsets = w->tile_offsets;
     a.tile_order = w->tile_order;
     a.gids = w->gids;

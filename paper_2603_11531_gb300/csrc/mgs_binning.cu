@@ -4,10 +4,10 @@
 // (Sec. 2, Eq. 1 discussion; Sec. 3.1).  The lists built here are keyed by
 // tile only -- a counting sort by tile:
 //
-//   0. k_group_cost, k_bin_plan: the plan cost of every group of 32
-//      consecutive Gaussians (its rectangle rows, each charged kRowCost plus
-//      the row's width in tiles) and the exclusive scan of the group costs
-//      plus a fixed visit charge.  Every warp of the binning grid (one
+//   0. k_bin_plan: the exclusive scan of the groups' plan costs (a group is 32
+//      consecutive Gaussians; preprocessing has summed the costs of its
+//      rectangle rows, kRowCost plus the row's width in tiles each) plus a
+//      fixed visit charge.  Every warp of the binning grid (at most one
 //      512-thread CTA per SM) takes an equal contiguous share of that cost
 //      numbering, cut at row boundaries.
 //   1. k_bin_count: each warp resolves its rows, 32 at a time (one per lane):
@@ -283,10 +283,8 @@ __device__ __forceinline__ bool row_tiles(float mx, float my, float l11, float l
     return true;
 }
 
-// Plan cost of a rectangle row: kRowCost plus one unit per tile of the row.
-// The count resolves a row in about the same time whatever its width; the
-// scatter also writes the row's listed tiles (about 0.6 of its width).
-constexpr int kRowCost = 3;
+// Plan cost of a rectangle row: kRowCost plus its width, summed per group by
+// preprocessing.
 // Cost of a group in the work plan beyond its rows: a fixed charge for
 // visiting it (loading its 32 rectangles, the scans and the row split), so
 // that shares over sparse stretches of the scene (many Gaussians with one
@@ -425,14 +423,19 @@ __device__ __forceinline__ void warp_rows(const GroupLoad &L, int64_t g0, int ca
     }
 }
 
-// Largest group g with cexcl[g] <= c (c < cexcl[groups]).
+// Largest group g with cexcl[g] <= c (c < cexcl[groups]); the warp probes 32
+// entries at a time (three dependent loads for 18,750 groups instead of the
+// fifteen of a binary search, about 4 us of the count and of the scatter).
 __device__ __forceinline__ int64_t find_group(const unsigned long long *__restrict__ cexcl,
                                               int64_t groups, unsigned long long c) {
-    int64_t lo = 0, hi = groups - 1;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) >> 1;
-        if (cexcl[mid] <= c) lo = mid;
-        else hi = mid - 1;
+    const int lane = threadIdx.x & 31;
+    int64_t lo = 0, hi = groups;   // cexcl[lo] <= c < cexcl[hi]
+    while (hi - lo > 1) {
+        const int64_t step = (hi - lo + 31) / 32;
+        const int64_t p = lo + step * (lane + 1);
+        const unsigned le = __ballot_sync(0xffffffffu, p < hi && cexcl[p] <= c);
+        lo += step * __popc(le);
+        if (lo + step < hi) hi = lo + step;
     }
     return lo;
 }
@@ -488,22 +491,6 @@ __device__ __forceinline__ void warp_share_rows(const uint2 *__restrict__ rect,
         if (done) break;
     }
     if (qn > 0) run_rows(q, qh, qn, f);
-}
-
-// Plan cost of every group of 32 consecutive Gaussians: the sum of
-// h (kRowCost + w) over its rectangles (one warp per group).
-__global__ void __launch_bounds__(kBinThreads) k_group_cost(const uint2 *__restrict__ rect,
-                                                            int64_t n, uint32_t *__restrict__ grp) {
-    const int64_t g = ((int64_t)blockIdx.x * kBinThreads + threadIdx.x) >> 5;
-    const int64_t i = g * 32 + (threadIdx.x & 31);
-    uint32_t c = 0;
-    if (i < n) {
-        int x0, y0, w, h;
-        rect_of(rect[i], x0, y0, w, h);
-        c = (w > 0 && h > 0) ? (uint32_t)(h * (kRowCost + w)) : 0u;
-    }
-    c = __reduce_add_sync(0xffffffffu, c);
-    if ((threadIdx.x & 31) == 0 && g * 32 < n) grp[g] = c;
 }
 
 // Exclusive scan of the group costs (plus kGroupCost) into cexcl[0..groups]
@@ -821,14 +808,23 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_order(const uint32_t *__r
 
 }  // namespace
 
-// One binning CTA per SM at most (one per 1024 Gaussians below that): the
-// work plan balances the warps, so a second resident CTA would only add
-// per-CTA tile bases.
+// One binning CTA per SM at most: the work plan balances the warps, so a second
+// resident CTA would only add per-CTA tile bases.  Below that, one per 512
+// Gaussians, a group per warp: small scenes are bound by the latency of a warp's
+// walk over its groups (50k frame at 640x480 77 us against 83 us with one CTA
+// per 1024 Gaussians; 4k frame 53 against 60 us), while views served together
+// prefer few CTAs (twelve views of 40k to 160k: 1.08 ms, 1.05 with one per 1024,
+// 1.10 with one per 256).
 int bin_ctas(int64_t n, int sm_count) {
-    int64_t c = (n + 1023) / 1024;
+    int64_t c = (n + 511) / 512;
     const int64_t cap = (int64_t)sm_count;
     if (c > cap) c = cap;
     return c < 1 ? 1 : (int)c;
+}
+
+uint32_t *bin_group_cost(uint32_t *scratch, int64_t n, int64_t T, int sm_count) {
+    const int64_t groups = (n + 31) / 32;
+    return scratch + (bin_ctas(n, sm_count) * T + 1) / 2 * 2 + 2 * (groups + 1);
 }
 
 int64_t bin_scratch_words(int64_t n, int64_t T, int sm_count) {
@@ -844,11 +840,12 @@ cudaError_t launch_binning(const RenderArgs &a, int sm_count, uint32_t *scratch,
     uint32_t *bases = scratch;
     unsigned long long *excl =
         reinterpret_cast<unsigned long long *>(scratch + ((int64_t)C * T + 1) / 2 * 2);
-    uint32_t *grp = reinterpret_cast<uint32_t *>(excl + groups + 1);
     const int brows = band_rows(tx, ty);
     const size_t count_smem = ((size_t)brows * (tx + 1) * sizeof(int) + (size_t)brows * tx + 15) / 16 * 16;
     const size_t scatter_smem = (size_t)brows * tx * sizeof(uint32_t);
-    cudaError_t e = cudaMemsetAsync(a.tile_count, 0, (size_t)T * sizeof(uint32_t), stream);
+    cudaError_t e = cudaSuccess;
+    if (a.n == 0)   // preprocessing, which clears the counts, did not run
+        e = cudaMemsetAsync(a.tile_count, 0, (size_t)T * sizeof(uint32_t), stream);
     if (e != cudaSuccess) return e;
     if (a.n > 0) {
         if ((e = cudaFuncSetAttribute(k_bin_count, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -857,15 +854,12 @@ cudaError_t launch_binning(const RenderArgs &a, int sm_count, uint32_t *scratch,
         if ((e = cudaFuncSetAttribute(k_bin_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)(kBand * sizeof(uint32_t)))) != cudaSuccess)
             return e;
-        k_group_cost<<<(int)((groups * 32 + kBinThreads - 1) / kBinThreads), kBinThreads, 0,
-                       stream>>>(a.rect, a.n, grp);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
         const int plan_n = (int)(groups < kPlanSeg ? groups : kPlanSeg);
         const size_t plan_smem = (size_t)(plan_n + plan_n / 16) * sizeof(unsigned long long);
         if ((e = cudaFuncSetAttribute(k_bin_plan, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)(kPlanSlots * sizeof(unsigned long long)))) != cudaSuccess)
             return e;
-        k_bin_plan<<<1, kScanThreads, plan_smem, stream>>>(grp, groups, excl);
+        k_bin_plan<<<1, kScanThreads, plan_smem, stream>>>(a.group_cost, groups, excl);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (marks && (e = cudaEventRecord(marks[0], stream)) != cudaSuccess) return e;
         k_bin_count<<<C, kBinThreads, count_smem, stream>>>(a.rect, a.rec, a.n, tx, ty, excl, groups,

@@ -145,6 +145,7 @@ struct RenderArgs {
     ProjRec *rec;
     uint2 *rect;              // packed (x_lo | x_hi << 16, y_lo | y_hi << 16 | kRectWide)
     uint32_t *tile_count;     // [T]
+    uint32_t *group_cost;     // [ceil(n / 32)] plan costs of binning (kRowCost), written by preprocessing
     uint32_t *tile_offsets;   // [T + 1]
     uint32_t *tile_order;     // [T] rasterisation order (longest lists first), | kTileWide
     uint32_t *gids;           // [capacity]
@@ -159,6 +160,13 @@ struct RenderArgs {
     int32_t *out_count;
     float *out_depth;          // depth image (Eq. 5), optional
 };
+
+// Plan cost of a rectangle row in binning: kRowCost plus one unit per tile of
+// the row.  The count resolves a row in about the same time whatever its width;
+// the scatter also writes the row's listed tiles (about 0.6 of its width).
+// Preprocessing, whose warps each hold the 32 Gaussians of a binning group,
+// sums the costs of a group's rows.
+constexpr int kRowCost = 3;
 
 // Does this render rasterise with tensor-core sums (FP16 attributes, no
 // comparator, not forced onto the FMA pipe)?  Preprocessing then also writes
@@ -249,14 +257,16 @@ cudaError_t launch_sorted(const RenderArgs &a, const SortedScratch &s, cudaStrea
 
 // Launchers (each enqueues its kernels on `stream`).
 cudaError_t launch_preprocess(const RenderArgs &a, int sm_count, cudaStream_t stream);
-// Per-tile counts, scan and scatter.  `scratch` has bin_scratch_words(n, T,
-// sm_count) 32-bit words: the per-CTA tile bases, then the pair counts of the
-// 32-Gaussian groups and their exclusive scan.
-// marks (nullable): three events recorded on `stream` after the plan (count
-// reset, group pairs, plan scan), after the count and after the tile scan.
+// Per-tile counts, scan and scatter, after launch_preprocess (which clears the
+// tile counts and writes the group costs).  `scratch` has bin_scratch_words(n,
+// T, sm_count) 32-bit words: the per-CTA tile bases, then the scan of the
+// 32-Gaussian groups' costs and (at bin_group_cost()) the costs.
+// marks (nullable): three events recorded on `stream` after the plan scan,
+// after the count and after the tile scan.
 cudaError_t launch_binning(const RenderArgs &a, int sm_count, uint32_t *scratch, cudaStream_t stream,
                            const cudaEvent_t *marks = nullptr);
 int bin_ctas(int64_t n, int sm_count);
+uint32_t *bin_group_cost(uint32_t *scratch, int64_t n, int64_t T, int sm_count);
 __host__ __device__ constexpr int64_t bin_scratch_words_for(int64_t ctas, int64_t T, int64_t n) {
     return (ctas * T + 1) / 2 * 2 + 2 * ((n + 31) / 32 + 1) + (n + 31) / 32;
 }

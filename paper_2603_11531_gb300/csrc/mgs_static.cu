@@ -26,7 +26,7 @@ using namespace mgs;
 constexpr int64_t kMaxGaussians = 131072;
 constexpr int kMaxTiles = 8192;
 constexpr int64_t kMaxPairs = int64_t(1) << 22;
-constexpr int kMaxBinCtas = (int)((kMaxGaussians + 1023) / 1024);  // bin_ctas() bound
+constexpr int kMaxBinCtas = 128;   // binning CTAs: the SM count, at most this
 
 constexpr size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 constexpr size_t kRecOff = 0;
@@ -143,12 +143,14 @@ extern "C" mgs_status mgs_render_static(const void *attrs, int64_t n, int32_t pr
     a.status = reinterpret_cast<DevStatus *>(S + kStatusOff);
     a.out_rgb = out_rgb;
     uint32_t *bases = reinterpret_cast<uint32_t *>(S + kBasesOff);
+    const int bin_sms = sm_count < kMaxBinCtas ? sm_count : kMaxBinCtas;
+    a.group_cost = bin_group_cost(bases, n, (int64_t)tiles_x * tiles_y, bin_sms);
 
     // the array keeps the previous call's contents: clear what starts at zero
-    // (tile counts are cleared by the binning launch itself)
+    // (tile counts are cleared by preprocessing)
     cudaError_t e = cudaMemsetAsync(a.status, 0, sizeof(DevStatus), stream);
     if (e == cudaSuccess && n > 0) e = launch_preprocess(a, sm_count, stream);
-    if (e == cudaSuccess) e = launch_binning(a, sm_count, bases, stream);
+    if (e == cudaSuccess) e = launch_binning(a, bin_sms, bases, stream);
     if (e == cudaSuccess) e = launch_raster(a, stream);
     DevStatus h{};
     if (e == cudaSuccess)
