@@ -157,8 +157,21 @@ mgs_status mgs_ctx_info(mgs_ctx ctx, int32_t *sm_count, int64_t *free_bytes,
  * gradients) uses the caller's indices. */
 mgs_status mgs_load_scene(mgs_ctx ctx, const mgs_scene_desc *desc,
                           mgs_stream stream, mgs_scene *out);
+/* A scene over the caller's device memory, for programs whose parameters
+ * change with every render (training): nothing is allocated, and the call is
+ * asynchronous on `stream`.  attrs (n x 24 elements of `precision`, 16-byte
+ * aligned) and mlp_blob (mgs_mlp_blob_bytes() bytes, 16-byte aligned) must stay
+ * valid and unchanged until the scene's last use on the device; the Gaussians
+ * keep the given order.  mlp: six device FP32 arrays w1 [64][22], b1 [64],
+ * w2 [64][64], b2 [64], w3 [5][64], b3 [5], rounded to BF16 (weights) and packed
+ * into mlp_blob; NULL: no MLP (mlp_blob unused).  mgs_unload_scene releases the
+ * handle. */
+mgs_status mgs_borrow_scene(mgs_ctx ctx, int64_t n, int32_t precision, const void *attrs,
+                            const float *const mlp[6], void *mlp_blob, mgs_stream stream,
+                            mgs_scene *out);
+int64_t mgs_mlp_blob_bytes(void);
 mgs_status mgs_unload_scene(mgs_scene scene);
-/* Device bytes held by the scene. */
+/* Device bytes held by the scene (0 for a borrowed one). */
 int64_t mgs_scene_bytes(mgs_scene scene);
 
 /* ---- workspaces (per-frame scratch) -------------------------------------- */

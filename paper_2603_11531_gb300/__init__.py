@@ -40,7 +40,7 @@ MGS_ORDER_AS_GIVEN = 2
 # Every entry point declared in include/mobilegs.h.
 EXPORTS = (
     "mgs_ctx_create", "mgs_ctx_destroy", "mgs_ctx_info", "mgs_load_scene",
-    "mgs_unload_scene", "mgs_scene_bytes", "mgs_workspace_create", "mgs_workspace_destroy",
+    "mgs_borrow_scene", "mgs_mlp_blob_bytes", "mgs_unload_scene", "mgs_scene_bytes", "mgs_workspace_create", "mgs_workspace_destroy",
     "mgs_workspace_reserve", "mgs_workspace_bytes", "mgs_workspace_sync", "mgs_render",
     "mgs_render_checked", "mgs_render_to_host", "mgs_tile_lists", "mgs_last_error",
     "mgs_version", "mgs_workspace_set_timing", "mgs_workspace_stage_times",
@@ -101,6 +101,8 @@ def lib():
                 "mgs_ctx_destroy": ([P], I32),
                 "mgs_ctx_info": ([P, ctypes.POINTER(I32), ctypes.POINTER(I64), ctypes.POINTER(I64)], I32),
                 "mgs_load_scene": ([P, ctypes.POINTER(mgs_scene_desc), P, PP], I32),
+                "mgs_borrow_scene": ([P, I64, I32, P, ctypes.POINTER(P), P, P, PP], I32),
+                "mgs_mlp_blob_bytes": ([], I64),
                 "mgs_unload_scene": ([P], I32),
                 "mgs_scene_bytes": ([P], I64),
                 "mgs_workspace_create": ([P, PP], I32),
@@ -227,12 +229,8 @@ def _check_render_outputs(ws, cam, out_rgb, out_aux=None, out_count=None, out_de
 
 def camera_struct(cam) -> mgs_camera:
     c = mgs_camera()
-    R = np.asarray(cam.R, np.float32).reshape(9)
-    t = np.asarray(cam.t, np.float32).reshape(3)
-    for i in range(9):
-        c.R[i] = float(R[i])
-    for i in range(3):
-        c.t[i] = float(t[i])
+    c.R[:] = np.asarray(cam.R, np.float32).reshape(9).tolist()
+    c.t[:] = np.asarray(cam.t, np.float32).reshape(3).tolist()
     c.fx, c.fy, c.cx, c.cy = (float(v) for v in (cam.fx, cam.fy, cam.cx, cam.cy))
     c.width, c.height = int(cam.width), int(cam.height)
     c.znear = float(getattr(cam, "znear", 0.2))
@@ -314,6 +312,37 @@ def mgs_load_scene(ctx, attrs, mlp=None, stream=None, order=MGS_ORDER_AUTO):
     h = ctypes.c_void_p()
     _check(lib().mgs_load_scene(ctx, ctypes.byref(d), _stream(stream, dev), ctypes.byref(h)))
     _scene_info[h.value] = (dev, d.n)
+    return h
+
+
+def mgs_mlp_blob_bytes() -> int:
+    return lib().mgs_mlp_blob_bytes()
+
+
+def mgs_borrow_scene(ctx, attrs, mlp=None, mlp_blob=None, stream=None):
+    """Scene over the caller's tensors (see include/mobilegs.h): attrs (N, 24)
+    float32/float16, mlp six float32 tensors (w1, b1, w2, b2, w3, b3) or None,
+    mlp_blob a uint8 tensor of mgs_mlp_blob_bytes(); all contiguous CUDA tensors
+    on the context's device, kept alive and unchanged by the caller."""
+    import torch
+    dev = _dev_of(ctx, _ctx_dev, "context")
+    if attrs.ndim != 2 or attrs.shape[1] != 24:
+        raise ValueError("attrs must have shape (N, 24)")
+    if attrs.dtype not in (torch.float16, torch.float32):
+        raise TypeError("attrs must be float16 or float32")
+    _check_dev_tensor(attrs, tuple(attrs.shape), attrs.dtype, dev, "attrs")
+    ptrs = None
+    if mlp is not None:
+        for t, shape, what in zip(mlp, ((64, 22), (64,), (64, 64), (64,), (5, 64), (5,)),
+                                  ("w1", "b1", "w2", "b2", "w3", "b3"), strict=True):
+            _check_dev_tensor(t, shape, torch.float32, dev, what)
+        _check_dev_tensor(mlp_blob, (mgs_mlp_blob_bytes(),), torch.uint8, dev, "mlp_blob")
+        ptrs = (ctypes.c_void_p * 6)(*[t.data_ptr() for t in mlp])
+    prec = MGS_PREC_FP16 if attrs.dtype == torch.float16 else MGS_PREC_FP32
+    h = ctypes.c_void_p()
+    _check(lib().mgs_borrow_scene(ctx, int(attrs.shape[0]), prec, _ptr(attrs), ptrs, _ptr(mlp_blob),
+                                  _stream(stream, dev), ctypes.byref(h)))
+    _scene_info[h.value] = (dev, int(attrs.shape[0]))
     return h
 
 

@@ -3,20 +3,27 @@
 Training-style use: Gaussian attributes (N, 24) and, optionally, the MLP
 parameters are CUDA tensors that require grad.  Every step of the forward and
 backward runs in the library's kernels; this module only moves tensors across
-the C-ABI (the MLP weights are rounded to BF16 bit patterns for the tensor
-cores on the way in).
+the C-ABI.  The parameters of a step change before the next one, so a step's
+scene is borrowed device memory (a copy of the attributes and the MLP packed to
+BF16, both from torch's allocator) instead of a loaded scene: uploading the MLP
+through the host and allocating and freeing device memory took 1.0 ms of a
+step, whatever its size.
 """
 from __future__ import annotations
 
 import numpy as np
 import torch
 
-from . import (MLP_GRAD_SIZE, Renderer, mgs_load_scene, mgs_render_checked, mgs_render_backward,
-               mgs_unload_scene, render_opts)
+from . import (MLP_GRAD_SIZE, Renderer, camera_struct, mgs_borrow_scene, mgs_camera, mgs_load_scene,
+               mgs_mlp_blob_bytes, mgs_render_backward, mgs_render_checked, mgs_unload_scene,
+               render_opts)
 from .synth import MLPWeights, f32_to_bf16_bits
 
 _SHAPES = (("w1", (64, 22)), ("b1", (64,)), ("w2", (64, 64)), ("b2", (64,)),
            ("w3", (5, 64)), ("b3", (5,)))
+_SIZES = [int(np.prod(shp)) for _, shp in _SHAPES]
+# mgs_load_scene stores larger scenes in spatial order, which pays there
+_MAX_BORROWED = 1 << 21
 
 
 def _mlp_from_tensors(ts) -> MLPWeights:
@@ -26,15 +33,38 @@ def _mlp_from_tensors(ts) -> MLPWeights:
                       f32_to_bf16_bits(arr[4]), arr[5].astype(np.float32))
 
 
+def _step_scene(renderer, attrs, mlp):
+    """The scene of one step and the tensors it borrows."""
+    if attrs.ndim == 2 and attrs.shape[0] > _MAX_BORROWED:
+        return mgs_load_scene(renderer.ctx, attrs.detach().contiguous(),
+                              _mlp_from_tensors(mlp) if mlp else None), ()
+    a = attrs.detach().clone(memory_format=torch.contiguous_format)
+    params = blob = None
+    if mlp:
+        params = [t if t.dtype == torch.float32 and t.device == a.device and t.is_contiguous()
+                  else t.detach().to(device=a.device, dtype=torch.float32).contiguous() for t in mlp]
+        blob = torch.empty(mgs_mlp_blob_bytes(), dtype=torch.uint8, device=a.device)
+    return mgs_borrow_scene(renderer.ctx, a, params, blob), (a, blob)
+
+
+def _after_last_backward(renderer, stream):
+    """Orders `stream` after the renderer's last backward, which returns before
+    its kernels are done with the renderer's workspace."""
+    last = getattr(renderer, "_backward_done", None)
+    if last is not None and last[0] != stream:
+        stream.wait_event(last[1])
+
+
 class RenderFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, renderer, cam, opts, attrs, *mlp):
-        mlpw = _mlp_from_tensors(mlp) if mlp else None
-        scene = mgs_load_scene(renderer.ctx, attrs.detach().contiguous(), mlpw)
-        H, W = int(cam.height), int(cam.width)
-        rgb = torch.empty((H, W, 3), dtype=torch.float32, device=attrs.device)
-        aux = torch.empty((5, H, W), dtype=torch.float32, device=attrs.device)
+        scene, ctx.borrowed = _step_scene(renderer, attrs, mlp)
         try:
+            cam = cam if isinstance(cam, mgs_camera) else camera_struct(cam)
+            H, W = cam.height, cam.width
+            rgb = torch.empty((H, W, 3), dtype=torch.float32, device=attrs.device)
+            aux = torch.empty((5, H, W), dtype=torch.float32, device=attrs.device)
+            _after_last_backward(renderer, torch.cuda.current_stream(renderer.device))
             mgs_render_checked(renderer.ws, scene, cam, opts, rgb, aux)
         except Exception:
             mgs_unload_scene(scene)
@@ -48,22 +78,28 @@ class RenderFn(torch.autograd.Function):
     @staticmethod
     def backward(ctx, g):
         (aux,) = ctx.saved_tensors
+        if ctx.scene is None:
+            raise ValueError("the scene of this render was released by its first backward")
         dev = aux.device
         d_attrs = torch.empty(ctx.attrs_shape, dtype=torch.float32, device=dev)
         d_mlp = torch.empty(MLP_GRAD_SIZE, dtype=torch.float32, device=dev) if ctx.n_mlp else None
+        stream = torch.cuda.current_stream(dev)
         try:
+            _after_last_backward(ctx.renderer, stream)
             mgs_render_backward(ctx.renderer.ws, ctx.scene, ctx.cam, ctx.opts, g.contiguous(), aux,
                                 d_attrs, d_mlp)
-            torch.cuda.synchronize(dev)
+            if ctx.borrowed:
+                done = torch.cuda.Event()
+                done.record(stream)
+                ctx.renderer._backward_done = (stream, done)
+            else:   # the library frees the scene's memory
+                torch.cuda.synchronize(dev)
         finally:
             mgs_unload_scene(ctx.scene)
+            ctx.scene = None
         grads = [None, None, None, d_attrs.to(ctx.attrs_dtype)]
         if ctx.n_mlp:
-            off = 0
-            for _, shp in _SHAPES:
-                k = int(np.prod(shp))
-                grads.append(d_mlp[off:off + k].view(shp))
-                off += k
+            grads += [t.view(shp) for t, (_, shp) in zip(d_mlp.split(_SIZES), _SHAPES)]
         return tuple(grads)
 
 

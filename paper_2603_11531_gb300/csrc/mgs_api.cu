@@ -75,6 +75,7 @@ struct mgs_scene_s {
     int precision = MGS_PREC_FP32;
     void *attrs = nullptr;
     bool has_mlp = false;
+    bool borrowed = false;              // attrs and the MLP blob are the caller's memory
     unsigned char *mlp_blob = nullptr;  // packed weights + biases
     DevMLP mlp{};
     uint32_t *perm = nullptr;    // stored row -> caller index (spatial order)
@@ -109,6 +110,7 @@ struct mgs_workspace_s {
     SortedScratch ss{};            // sorted comparator scratch
     int64_t ss_n_cap = 0, ss_pairs_cap = 0, ss_tiles_cap = 0;
     DevStatus *status = nullptr;
+    DevStatus *status_host = nullptr;      // pinned copy, read by mgs_workspace_sync
     int64_t last_tiles = 0;
     const uint32_t *last_perm = nullptr;   // storage -> caller order of the last scene
     uint64_t grow_hint = 0;  // pairs needed by an overflowed render
@@ -183,6 +185,10 @@ mgs_status ws_ensure(mgs_workspace_s *w, int64_t n, int64_t tiles, uint64_t pair
         if ((e = dev_alloc(&w->status, 1)) != cudaSuccess) return cuda_fail(e, "workspace");
         if ((e = cudaMemset(w->status, 0, sizeof(DevStatus))) != cudaSuccess)
             return cuda_fail(e, "workspace");
+        if ((e = cudaMallocHost(&w->status_host, sizeof(DevStatus))) != cudaSuccess) {
+            dev_free(w->status);
+            return cuda_fail(e, "workspace");
+        }
     }
     return MGS_OK;
 }
@@ -555,37 +561,27 @@ mgs_status mgs_load_scene(mgs_ctx ctx, const mgs_scene_desc *d, mgs_stream strea
         s->has_mlp = true;
         s->bytes += (int64_t)total;
     } else if (e == cudaSuccess && all_mlp) {
-        // pack: w1 [64][32] (cols 22.. zero), w2 [64][64], w3 [8][64] (rows 5.. zero)
-        const size_t n_w1 = kMlpHidden * kMlpK1, n_w2 = kMlpHidden * kMlpHidden,
-                     n_w3 = kMlpN3 * kMlpHidden;
-        const size_t off_w2 = n_w1 * 2, off_w3 = off_w2 + n_w2 * 2, off_b1 = off_w3 + n_w3 * 2,
-                     off_b2 = off_b1 + 64 * 4, off_b3 = off_b2 + 64 * 4, total = off_b3 + 8 * 4;
-        std::vector<unsigned char> blob(total, 0);
+        std::vector<unsigned char> blob(kBlobBytes, 0);
         uint16_t *w1 = reinterpret_cast<uint16_t *>(blob.data());
-        uint16_t *w2 = reinterpret_cast<uint16_t *>(blob.data() + off_w2);
-        uint16_t *w3 = reinterpret_cast<uint16_t *>(blob.data() + off_w3);
-        float *b1 = reinterpret_cast<float *>(blob.data() + off_b1);
-        float *b2 = reinterpret_cast<float *>(blob.data() + off_b2);
-        float *b3 = reinterpret_cast<float *>(blob.data() + off_b3);
+        uint16_t *w2 = reinterpret_cast<uint16_t *>(blob.data() + kBlobW2);
+        uint16_t *w3 = reinterpret_cast<uint16_t *>(blob.data() + kBlobW3);
+        float *b1 = reinterpret_cast<float *>(blob.data() + kBlobB1);
+        float *b2 = reinterpret_cast<float *>(blob.data() + kBlobB2);
+        float *b3 = reinterpret_cast<float *>(blob.data() + kBlobB3);
         for (int r = 0; r < kMlpHidden; ++r)
             for (int c = 0; c < kMlpIn; ++c) w1[r * kMlpK1 + c] = d->mlp_w1[r * kMlpIn + c];
-        memcpy(w2, d->mlp_w2, n_w2 * 2);
+        memcpy(w2, d->mlp_w2, (size_t)kMlpHidden * kMlpHidden * 2);
         memcpy(w3, d->mlp_w3, (size_t)kMlpOut * kMlpHidden * 2);
         memcpy(b1, d->mlp_b1, 64 * 4);
         memcpy(b2, d->mlp_b2, 64 * 4);
         memcpy(b3, d->mlp_b3, kMlpOut * 4);
-        e = cudaMalloc(&s->mlp_blob, total);
+        e = cudaMalloc(&s->mlp_blob, kBlobBytes);
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(s->mlp_blob, blob.data(), total, cudaMemcpyHostToDevice, stream);
+            e = cudaMemcpyAsync(s->mlp_blob, blob.data(), kBlobBytes, cudaMemcpyHostToDevice, stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-        s->mlp.w1 = reinterpret_cast<const __nv_bfloat16 *>(s->mlp_blob);
-        s->mlp.w2 = reinterpret_cast<const __nv_bfloat16 *>(s->mlp_blob + off_w2);
-        s->mlp.w3 = reinterpret_cast<const __nv_bfloat16 *>(s->mlp_blob + off_w3);
-        s->mlp.b1 = reinterpret_cast<const float *>(s->mlp_blob + off_b1);
-        s->mlp.b2 = reinterpret_cast<const float *>(s->mlp_blob + off_b2);
-        s->mlp.b3 = reinterpret_cast<const float *>(s->mlp_blob + off_b3);
+        s->mlp = blob_mlp(s->mlp_blob);
         s->has_mlp = true;
-        s->bytes += (int64_t)total;
+        s->bytes += (int64_t)kBlobBytes;
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) {
@@ -600,8 +596,53 @@ mgs_status mgs_load_scene(mgs_ctx ctx, const mgs_scene_desc *d, mgs_stream strea
     return MGS_OK;
 }
 
+int64_t mgs_mlp_blob_bytes(void) { return (int64_t)kBlobBytes; }
+
+mgs_status mgs_borrow_scene(mgs_ctx ctx, int64_t n, int32_t precision, const void *attrs,
+                            const float *const mlp[6], void *mlp_blob, mgs_stream stream_,
+                            mgs_scene *out) {
+    cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
+    if (!ctx || !out) return fail(MGS_ERR_INVALID_ARG, "NULL argument");
+    *out = nullptr;
+    if (n < 0 || n > (int64_t)1 << 31)
+        return fail(MGS_ERR_INVALID_ARG, "n = %lld outside 0..2^31", (long long)n);
+    if (precision != MGS_PREC_FP32 && precision != MGS_PREC_FP16)
+        return fail(MGS_ERR_INVALID_ARG, "unknown precision %d", precision);
+    if (n > 0 && !attrs) return fail(MGS_ERR_INVALID_ARG, "attrs is NULL");
+    if (reinterpret_cast<uintptr_t>(attrs) & 15)
+        return fail(MGS_ERR_INVALID_ARG, "device attrs must be 16-byte aligned");
+    if (mlp) {
+        for (int k = 0; k < 6; ++k)
+            if (!mlp[k]) return fail(MGS_ERR_INVALID_ARG, "MLP weights are partially given");
+        if (!mlp_blob || (reinterpret_cast<uintptr_t>(mlp_blob) & 15))
+            return fail(MGS_ERR_INVALID_ARG, "mlp_blob must be a 16-byte aligned device pointer");
+    }
+    DeviceGuard g(ctx->device);
+    if (!g.ok) return fail(MGS_ERR_CUDA, "cannot select device %d", ctx->device);
+    if (mlp) {
+        const cudaError_t e = launch_pack_mlp(mlp, mlp_blob, stream);
+        if (e != cudaSuccess) return cuda_fail(e, "MLP pack launch");
+    }
+    mgs_scene s = new mgs_scene_s;
+    s->ctx = ctx;
+    s->n = n;
+    s->precision = precision;
+    s->attrs = const_cast<void *>(attrs);
+    s->borrowed = true;
+    if (mlp) {
+        s->mlp = blob_mlp(static_cast<unsigned char *>(mlp_blob));
+        s->has_mlp = true;
+    }
+    *out = s;
+    return MGS_OK;
+}
+
 mgs_status mgs_unload_scene(mgs_scene s) {
     if (!s) return MGS_OK;
+    if (s->borrowed) {
+        delete s;
+        return MGS_OK;
+    }
     DeviceGuard g(s->ctx->device);
     cudaFree(s->attrs);
     dev_free(s->mlp_blob);
@@ -646,6 +687,7 @@ mgs_status mgs_workspace_destroy(mgs_workspace w) {
     dev_free(w->ss.vals_tmp);
     if (w->ss.temp) cudaFree(w->ss.temp);
     dev_free(w->status);
+    if (w->status_host) cudaFreeHost(w->status_host);
     for (auto &q : w->pending)
         for (auto x : q) cudaEventDestroy(x);
     for (auto x : w->event_pool) cudaEventDestroy(x);
@@ -669,15 +711,18 @@ mgs_status mgs_workspace_sync(mgs_workspace w, mgs_stream stream_, int64_t *pair
     cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
     if (!w) return fail(MGS_ERR_INVALID_ARG, "workspace is NULL");
     DeviceGuard g(w->ctx->device);
-    cudaError_t e = cudaStreamSynchronize(stream);
-    if (e != cudaSuccess) return cuda_fail(e, "stream synchronize");
+    // the status is read and reset in stream order: one wait for everything
+    cudaError_t e = cudaSuccess;
+    if (w->status) {
+        e = cudaMemcpyAsync(w->status_host, w->status, sizeof(DevStatus), cudaMemcpyDeviceToHost, stream);
+        if (e != cudaSuccess) return cuda_fail(e, "status read");
+        e = cudaMemsetAsync(w->status, 0, offsetof(DevStatus, last_pairs), stream);
+        if (e != cudaSuccess) return cuda_fail(e, "status reset");
+    }
+    if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return cuda_fail(e, "stream synchronize");
     if (pairs_out) *pairs_out = 0;
     if (!w->status) return MGS_OK;
-    DevStatus h;
-    if ((e = cudaMemcpy(&h, w->status, sizeof h, cudaMemcpyDeviceToHost)) != cudaSuccess)
-        return cuda_fail(e, "status read");
-    if ((e = cudaMemset(w->status, 0, offsetof(DevStatus, last_pairs))) != cudaSuccess)
-        return cuda_fail(e, "status reset");
+    const DevStatus h = *w->status_host;
     if (pairs_out) *pairs_out = (int64_t)h.max_pairs;
     if (h.overflow & kStatusMmaTimeout)
         return fail(MGS_ERR_TIMEOUT, "a tensor-core MMA wait in preprocessing timed out");

@@ -42,6 +42,26 @@ struct DevMLP {
     int h1, h2, h3;           // 0: the 22-64-64-5 MLP; else App. C's three hidden layers
 };
 
+// Layout of the 22-64-64-5 MLP's packed weights in device memory (byte offsets):
+// w1 [64][32] (columns 22.. zero), w2 [64][64], w3 [8][64] (rows 5.. zero) in BF16,
+// then b1 [64], b2 [64], b3 [8] in FP32.
+constexpr size_t kBlobW2 = (size_t)kMlpHidden * kMlpK1 * 2;
+constexpr size_t kBlobW3 = kBlobW2 + (size_t)kMlpHidden * kMlpHidden * 2;
+constexpr size_t kBlobB1 = kBlobW3 + (size_t)kMlpN3 * kMlpHidden * 2;
+constexpr size_t kBlobB2 = kBlobB1 + kMlpHidden * 4;
+constexpr size_t kBlobB3 = kBlobB2 + kMlpHidden * 4;
+constexpr size_t kBlobBytes = kBlobB3 + kMlpN3 * 4;
+inline DevMLP blob_mlp(unsigned char *blob) {
+    DevMLP m{};
+    m.w1 = reinterpret_cast<const __nv_bfloat16 *>(blob);
+    m.w2 = reinterpret_cast<const __nv_bfloat16 *>(blob + kBlobW2);
+    m.w3 = reinterpret_cast<const __nv_bfloat16 *>(blob + kBlobW3);
+    m.b1 = reinterpret_cast<const float *>(blob + kBlobB1);
+    m.b2 = reinterpret_cast<const float *>(blob + kBlobB2);
+    m.b3 = reinterpret_cast<const float *>(blob + kBlobB3);
+    return m;
+}
+
 // Shared-memory layout (byte offsets) of the wide (three hidden layer)
 // tcgen05 MLP, two 128-row tiles per step: BF16 operands in canonical K-major
 // layout (features x of both tiles, activations a0/a1 of the current tile,
@@ -249,6 +269,9 @@ cudaError_t radix_sort(uint64_t **k, uint32_t **v, uint64_t **kt, uint32_t **vt,
 // its inverse.  Synchronous.
 cudaError_t spatial_order(const void *attrs_in, int64_t n, int precision, void *attrs_out,
                           uint32_t *perm, uint32_t *iperm, cudaStream_t stream);
+// Packs six device FP32 arrays (w1, b1, w2, b2, w3, b3 of the 22-64-64-5 MLP) into
+// the blob that DevMLP's pointers address (mgs_preprocess.cu).
+cudaError_t launch_pack_mlp(const float *const mlp[6], void *blob, cudaStream_t stream);
 // out[j] = perm[in[j]] for j < count.
 cudaError_t map_ids(const uint32_t *in, const uint32_t *perm, int64_t count, uint32_t *out,
                     cudaStream_t stream);

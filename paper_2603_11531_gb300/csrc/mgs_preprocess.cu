@@ -370,7 +370,36 @@ cudaError_t launch_t(const RenderArgs &a, int sm_count, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
+// One thread per blob element; reads are coalesced, the whole MLP is 36 KB.
+__global__ void __launch_bounds__(256) k_pack_mlp(const float *__restrict__ w1, const float *__restrict__ b1,
+                                                  const float *__restrict__ w2, const float *__restrict__ b2,
+                                                  const float *__restrict__ w3, const float *__restrict__ b3,
+                                                  unsigned char *__restrict__ blob) {
+    __nv_bfloat16 *o1 = reinterpret_cast<__nv_bfloat16 *>(blob);
+    __nv_bfloat16 *o2 = reinterpret_cast<__nv_bfloat16 *>(blob + kBlobW2);
+    __nv_bfloat16 *o3 = reinterpret_cast<__nv_bfloat16 *>(blob + kBlobW3);
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < kMlpHidden * kMlpK1) {
+        const int r = e / kMlpK1, c = e % kMlpK1;
+        o1[e] = __float2bfloat16_rn(c < kMlpIn ? w1[r * kMlpIn + c] : 0.0f);
+    }
+    if (e < kMlpHidden * kMlpHidden) o2[e] = __float2bfloat16_rn(w2[e]);
+    if (e < kMlpN3 * kMlpHidden) o3[e] = __float2bfloat16_rn(e < kMlpOut * kMlpHidden ? w3[e] : 0.0f);
+    if (e < kMlpHidden) {
+        reinterpret_cast<float *>(blob + kBlobB1)[e] = b1[e];
+        reinterpret_cast<float *>(blob + kBlobB2)[e] = b2[e];
+    }
+    if (e < kMlpN3) reinterpret_cast<float *>(blob + kBlobB3)[e] = e < kMlpOut ? b3[e] : 0.0f;
+}
+
 }  // namespace
+
+cudaError_t launch_pack_mlp(const float *const m[6], void *blob, cudaStream_t stream) {
+    static_assert(kMlpHidden * kMlpHidden >= kMlpHidden * kMlpK1, "the grid covers every array");
+    k_pack_mlp<<<kMlpHidden * kMlpHidden / 256, 256, 0, stream>>>(m[0], m[1], m[2], m[3], m[4], m[5],
+                                                                  static_cast<unsigned char *>(blob));
+    return cudaGetLastError();
+}
 
 cudaError_t launch_preprocess(const RenderArgs &a, int sm_count, cudaStream_t stream) {
     const bool fp16 = a.precision == MGS_PREC_FP16;
