@@ -504,6 +504,7 @@ constexpr int kPlanSlots = kPlanSeg + kPlanSeg / 16;
 __global__ void __launch_bounds__(kScanThreads) k_bin_plan(const uint32_t *__restrict__ grp,
                                                            int64_t groups,
                                                            unsigned long long *__restrict__ cexcl) {
+    grid_wait();
     extern __shared__ unsigned long long seg[];
     __shared__ unsigned long long warp_sums[kScanThreads / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -546,6 +547,7 @@ __global__ void __launch_bounds__(kScanThreads) k_bin_plan(const uint32_t *__res
         for (int i = tid; i < m; i += kScanThreads) cexcl[s0 + i] = seg[plan_slot(i)];
         __syncthreads();
     }
+    grid_trigger();
     if (tid == 0) cexcl[groups] = carry;
 }
 
@@ -570,6 +572,8 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_bin_count(const uint2 *__res
                                                            uint32_t *__restrict__ bases,
                                                            const DevStatus *__restrict__ status,
                                                            bool tc) {
+    grid_wait();
+    grid_trigger();   // the dependent (the tile scan) is one CTA
     extern __shared__ int diff_s[];
     __shared__ RowSlot queue_s[kBinThreads / 32][kQueue];
     const int T = tiles_x * tiles_y;
@@ -643,6 +647,7 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_bin_scatter(
     const uint32_t *__restrict__ offsets, const uint32_t *__restrict__ bases,
     uint32_t *__restrict__ gids, uint64_t capacity, const DevStatus *__restrict__ status,
     const ProjRec *__restrict__ rec, uint4 *__restrict__ wt16) {
+    grid_wait();
     extern __shared__ uint32_t cur_s[];
     __shared__ RowSlot queue_s[kBinThreads / 32][kQueue];
     if (status->last_pairs > capacity) return;  // overflow: lists are not built
@@ -731,6 +736,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_order(const uint32_t *__r
                                                              uint32_t *__restrict__ offsets,
                                                              uint32_t *__restrict__ order, int T,
                                                              uint64_t capacity, DevStatus *status) {
+    grid_wait();
     __shared__ unsigned long long warp_sums[kScanThreads / 32];
     __shared__ unsigned long long carry;
     __shared__ uint32_t hist[33], start[33];
@@ -799,6 +805,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_order(const uint32_t *__r
         }
     }
     __syncthreads();
+    grid_trigger();
     for (int t = tid; t < T; t += blockDim.x) {
         const uint32_t cw = count[t], c = cw & kTileMask;
         order[atomicAdd(&start[c ? 32 - __clz(c) : 0], 1u)] = (uint32_t)t | (cw & kTileWide);
@@ -859,28 +866,27 @@ cudaError_t launch_binning(const RenderArgs &a, int sm_count, uint32_t *scratch,
         if ((e = cudaFuncSetAttribute(k_bin_plan, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)(kPlanSlots * sizeof(unsigned long long)))) != cudaSuccess)
             return e;
-        k_bin_plan<<<1, kScanThreads, plan_smem, stream>>>(a.group_cost, groups, excl);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_dependent(k_bin_plan, 1, kScanThreads, plan_smem, stream, a.group_cost, groups,
+                                  excl)) != cudaSuccess)
+            return e;
         if (marks && (e = cudaEventRecord(marks[0], stream)) != cudaSuccess) return e;
-        k_bin_count<<<C, kBinThreads, count_smem, stream>>>(a.rect, a.rec, a.n, tx, ty, excl, groups,
-                                                            a.tile_count, bases, a.status,
-                                                            tc_raster(a));
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_dependent(k_bin_count, C, kBinThreads, count_smem, stream, a.rect, a.rec, a.n, tx,
+                                  ty, excl, groups, a.tile_count, bases, a.status, tc_raster(a))) !=
+            cudaSuccess)
+            return e;
         if (marks && (e = cudaEventRecord(marks[1], stream)) != cudaSuccess) return e;
     } else if (marks) {
         if ((e = cudaEventRecord(marks[0], stream)) != cudaSuccess) return e;
         if ((e = cudaEventRecord(marks[1], stream)) != cudaSuccess) return e;
     }
-    k_scan_order<<<1, kScanThreads, 0, stream>>>(a.tile_count, a.tile_offsets, a.tile_order, T,
-                                                 a.capacity, a.status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_dependent(k_scan_order, 1, kScanThreads, 0, stream, a.tile_count, a.tile_offsets,
+                              a.tile_order, T, a.capacity, a.status)) != cudaSuccess)
+        return e;
     if (marks && (e = cudaEventRecord(marks[2], stream)) != cudaSuccess) return e;
     if (a.n == 0) return e;
-    k_bin_scatter<<<C, kBinThreads, scatter_smem, stream>>>(a.rect, a.n, tx, ty, excl, groups,
-                                                            a.tile_offsets, bases, a.gids,
-                                                            a.capacity, a.status, a.rec,
-                                                            tc_raster(a) ? a.wt16 : nullptr);
-    return cudaGetLastError();
+    return launch_dependent(k_bin_scatter, C, kBinThreads, scatter_smem, stream, a.rect, a.n, tx, ty, excl,
+                            groups, a.tile_offsets, bases, a.gids, a.capacity, a.status, a.rec,
+                            tc_raster(a) ? a.wt16 : nullptr);
 }
 
 }  // namespace mgs

@@ -6,10 +6,37 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <utility>
 
 #include "mobilegs.h"
 
 namespace mgs {
+
+// Kernels of a render are launched as programmatic dependents of their
+// predecessor in the stream: the launch is set up while the predecessor still
+// runs, and grid_wait(), the first statement of every such kernel, waits until
+// it has completed with its writes visible (so each kernel is ordered after all
+// earlier ones).  grid_trigger() lets the dependent's CTAs become resident
+// before the predecessor's last CTA has exited; it is called where the
+// dependent is a single CTA or the work is nearly done, so that waiting CTAs do
+// not hold registers that other streams could use.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
+                             cudaStream_t stream, A &&...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(std::forward<A>(args))...);
+}
 
 constexpr int kTile = 16;         // tile edge in pixels (binning granularity)
 constexpr int kRec = 24;          // stored elements per Gaussian

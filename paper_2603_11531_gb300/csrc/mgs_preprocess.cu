@@ -181,6 +181,8 @@ __global__ void __launch_bounds__(kWide ? tcw::kThreads : (kTC ? tc::kThreads : 
     k_preprocess(RenderArgs args) {
     constexpr int kStep =
         kWide ? tcw::kThreads : (kTC ? tc::kThreads : kThreads);   // Gaussians per CTA step
+    grid_wait();
+    grid_trigger();   // the dependent (the binning plan) is one CTA
     extern __shared__ __align__(128) unsigned char smem_raw[];
     MlpSmem &sm = *reinterpret_cast<MlpSmem *>(smem_raw);
     tc::Smem &tsm = *reinterpret_cast<tc::Smem *>(smem_raw);
@@ -346,8 +348,7 @@ cudaError_t launch_wide(const RenderArgs &a, int sm_count, cudaStream_t stream) 
     int64_t blocks = (a.n + tcw::kThreads - 1) / tcw::kThreads;
     if (blocks > sm_count) blocks = sm_count;
     if (blocks < 1) blocks = 1;
-    kern<<<(unsigned)blocks, tcw::kThreads, smem, stream>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(kern, (unsigned)blocks, tcw::kThreads, smem, stream, a);
 }
 
 template <bool kFP16, bool kMLP, bool kResidual, bool kTC>
@@ -366,8 +367,7 @@ cudaError_t launch_t(const RenderArgs &a, int sm_count, cudaStream_t stream) {
     const int64_t cap = (int64_t)sm_count * ((kMLP && kTC) ? 3 : 8);
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    kern<<<(unsigned)blocks, threads, smem, stream>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(kern, (unsigned)blocks, threads, smem, stream, a);
 }
 
 // One thread per blob element; reads are coalesced, the whole MLP is 36 KB.

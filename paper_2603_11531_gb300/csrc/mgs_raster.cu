@@ -820,6 +820,7 @@ __host__ __device__ __forceinline__ bool use_tc(const RenderArgs &a) { return tc
 // One CTA per tile, longest tile lists first.
 template <bool kAux, bool kCount, bool kDepth = false>
 __global__ void __launch_bounds__(kThreads) k_raster(RenderArgs args) {
+    grid_wait();
     __shared__ FmaSmem<kDepth> sm;
     if (args.status->last_pairs > args.capacity) return;  // overflowed: lists incomplete
     raster_tile<kAux, kCount, kDepth>(args, (int)(args.tile_order[blockIdx.x] & kTileMask), sm);
@@ -829,6 +830,7 @@ __global__ void __launch_bounds__(kThreads) k_raster(RenderArgs args) {
 // the others (kTileWide, see kWideWeight) take the FP32 FMA tile code.
 template <bool kAux, bool kCount, bool kDepth = false>
 __global__ void __launch_bounds__(kThreads) k_raster_tc(RenderArgs args) {
+    grid_wait();
     __shared__ union {
         TcSmem tc;
         ulonglong2 buf[2][kDepth ? 6 : 5][32];
@@ -885,10 +887,8 @@ template <bool kAux, bool kCount>
 cudaError_t launch_t(const RenderArgs &a, cudaStream_t stream) {
     const int T = a.cam.tiles_x * a.cam.tiles_y;
     if (use_tc(a))
-        k_raster_tc<kAux, kCount><<<T, kThreads, 0, stream>>>(a);
-    else
-        k_raster<kAux, kCount><<<T, kThreads, 0, stream>>>(a);
-    return cudaGetLastError();
+        return launch_dependent(k_raster_tc<kAux, kCount>, T, kThreads, 0, stream, a);
+    return launch_dependent(k_raster<kAux, kCount>, T, kThreads, 0, stream, a);
 }
 
 }  // namespace
@@ -896,11 +896,9 @@ cudaError_t launch_t(const RenderArgs &a, cudaStream_t stream) {
 cudaError_t launch_raster(const RenderArgs &a, cudaStream_t stream) {
     const bool aux = a.out_aux != nullptr, cnt = a.out_count != nullptr;
     if (a.out_depth) {   // depth image (Eq. 5), no aux / count outputs
-        if (use_tc(a))
-            k_raster_tc<false, false, true><<<a.cam.tiles_x * a.cam.tiles_y, kThreads, 0, stream>>>(a);
-        else
-            k_raster<false, false, true><<<a.cam.tiles_x * a.cam.tiles_y, kThreads, 0, stream>>>(a);
-        return cudaGetLastError();
+        const int T = a.cam.tiles_x * a.cam.tiles_y;
+        if (use_tc(a)) return launch_dependent(k_raster_tc<false, false, true>, T, kThreads, 0, stream, a);
+        return launch_dependent(k_raster<false, false, true>, T, kThreads, 0, stream, a);
     }
     if (aux && cnt) return launch_t<true, true>(a, stream);
     if (aux) return launch_t<true, false>(a, stream);
