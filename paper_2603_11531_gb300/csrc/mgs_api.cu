@@ -79,7 +79,7 @@ struct mgs_scene_s {
     unsigned char *mlp_blob = nullptr;  // packed weights + biases
     DevMLP mlp{};
     uint32_t *perm = nullptr;    // stored row -> caller index (spatial order)
-    uint32_t *iperm = nullptr;   // caller index -> stored row
+    uint32_t *iperm = nullptr;   // caller index -> stored row (behind perm, same allocation)
     int64_t bytes = 0;
 };
 
@@ -503,22 +503,25 @@ mgs_status mgs_load_scene(mgs_ctx ctx, const mgs_scene_desc *d, mgs_stream strea
     const bool spatial = d->n > 1 && (d->order == MGS_ORDER_SPATIAL ||
                                       (d->order == MGS_ORDER_AUTO && d->n > (int64_t(1) << 21)));
     cudaError_t e = cudaMalloc(&s->attrs, bytes ? bytes : 16);
-    if (e == cudaSuccess && spatial) e = cudaMalloc(&s->perm, (size_t)d->n * 4);
-    if (e == cudaSuccess && spatial) e = cudaMalloc(&s->iperm, (size_t)d->n * 4);
+    if (e == cudaSuccess && spatial) e = cudaMalloc(&s->perm, (size_t)d->n * 8);
+    if (spatial) s->iperm = s->perm + d->n;
     if (e != cudaSuccess) {
         dev_free(s->perm);
-        dev_free(s->iperm);
         if (s->attrs) cudaFree(s->attrs);
         delete s;
         return cuda_fail(e, "scene allocation");
     }
     const cudaMemcpyKind kind = d->attrs_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     if (bytes && spatial) {
-        // upload, then store in spatial (Morton) order
+        // stored in spatial (Morton) order: from the caller's device memory, or
+        // from an upload
         void *tmp = nullptr;
-        e = cudaMalloc(&tmp, bytes);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(tmp, d->attrs, bytes, kind, stream);
-        if (e == cudaSuccess) e = spatial_order(tmp, d->n, d->precision, s->attrs, s->perm, s->iperm, stream);
+        if (!d->attrs_on_device) {
+            e = cudaMalloc(&tmp, bytes);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(tmp, d->attrs, bytes, kind, stream);
+        }
+        if (e == cudaSuccess)
+            e = spatial_order(tmp ? tmp : d->attrs, d->n, d->precision, s->attrs, s->perm, s->iperm, stream);
         if (tmp) cudaFree(tmp);
     } else if (bytes) {
         e = cudaMemcpyAsync(s->attrs, d->attrs, bytes, kind, stream);
@@ -587,7 +590,6 @@ mgs_status mgs_load_scene(mgs_ctx ctx, const mgs_scene_desc *d, mgs_stream strea
     if (e != cudaSuccess) {
         dev_free(s->mlp_blob);
         dev_free(s->perm);
-        dev_free(s->iperm);
         cudaFree(s->attrs);
         delete s;
         return cuda_fail(e, "scene upload");
@@ -647,7 +649,6 @@ mgs_status mgs_unload_scene(mgs_scene s) {
     cudaFree(s->attrs);
     dev_free(s->mlp_blob);
     dev_free(s->perm);
-    dev_free(s->iperm);
     delete s;
     return MGS_OK;
 }

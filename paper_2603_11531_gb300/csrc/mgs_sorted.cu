@@ -2,7 +2,7 @@
 // compositing the paper removes (its "with sorting" baseline, Sec. 1 and
 // Table 3).  Same preprocessing, same tile lists and the same inclusion test
 // as the sort-free renderer; in addition every tile's list is ordered by view
-// depth with a project-written radix sort, and each pixel blends front to back
+// depth, and each pixel blends front to back
 //   C = sum_i c_i a_i T_i + T c_bg,  T_i = prod_{j<i} (1 - a_j),
 // stopping before the Gaussian that would bring T below 1e-4 (3DGS early
 // termination).
@@ -12,8 +12,7 @@
 // tile's list (a segment of the counting sort's output) is then sorted by
 // rank.  Both sorts are the CUDA library's (CUB) device radix / segmented
 // sorts, the kind of sort a sorted 3DGS renderer uses, so the comparison is
-// not made against a slow sort.  The project's own LSD radix sort below
-// serves the load-time spatial order.
+// not made against a slow sort.
 #include <cub/device/device_radix_sort.cuh>
 #include <cub/device/device_segmented_sort.cuh>
 
@@ -21,164 +20,6 @@
 
 namespace mgs {
 namespace {
-
-constexpr int kRsThreads = 256;
-constexpr int kRsItems = 8;
-constexpr int kRsTile = kRsThreads * kRsItems;  // keys per block
-constexpr int kRsBins = 16;                     // 4-bit digits
-
-__device__ __forceinline__ int64_t count_of(int64_t n, const unsigned long long *n_dev) {
-    if (!n_dev) return n;
-    const unsigned long long d = *n_dev;
-    return d < (unsigned long long)n ? (int64_t)d : n;
-}
-
-__global__ void __launch_bounds__(kRsThreads) k_rs_hist(const uint64_t *__restrict__ keys,
-                                                        int64_t n_max,
-                                                        const unsigned long long *n_dev,
-                                                        int shift, int nblocks,
-                                                        uint32_t *__restrict__ hist) {
-    __shared__ uint32_t h[kRsBins];
-    const int64_t n = count_of(n_max, n_dev);
-    if (threadIdx.x < kRsBins) h[threadIdx.x] = 0u;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRsTile;
-    for (int i = threadIdx.x; i < kRsTile; i += kRsThreads) {
-        const int64_t idx = base + i;
-        if (idx < n) atomicAdd(&h[(keys[idx] >> shift) & (kRsBins - 1)], 1u);
-    }
-    __syncthreads();
-    if (threadIdx.x < kRsBins) hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
-}
-
-// Exclusive scan of m uint32 values in place, one block.
-__global__ void __launch_bounds__(1024) k_rs_scan(uint32_t *__restrict__ v, int64_t m) {
-    __shared__ uint32_t warp_sums[32];
-    __shared__ uint32_t carry;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) carry = 0u;
-    __syncthreads();
-    for (int64_t base = 0; base < m; base += 1024 * 4) {
-        const int64_t i0 = base + (int64_t)tid * 4;
-        uint32_t x[4], local = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            x[k] = (i0 + k < m) ? v[i0 + k] : 0u;
-            local += x[k];
-        }
-        uint32_t incl = local;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (lane == 31) warp_sums[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            uint32_t s = warp_sums[lane];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
-                if (lane >= o) s += y;
-            }
-            warp_sums[lane] = s;
-        }
-        __syncthreads();
-        uint32_t run = carry + (incl - local) + (warp > 0 ? warp_sums[warp - 1] : 0u);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if (i0 + k < m) v[i0 + k] = run;
-            run += x[k];
-        }
-        __syncthreads();
-        if (tid == 1023) carry = run;
-        __syncthreads();
-    }
-}
-
-// Stable scatter of one 4-bit digit: thread t owns keys [8t, 8t + 8) of the
-// block; ranks = global digit offset + counts of the digit in earlier threads
-// + earlier keys of the same digit in this thread.
-__global__ void __launch_bounds__(kRsThreads) k_rs_scatter(
-    const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin,
-    uint64_t *__restrict__ kout, uint32_t *__restrict__ vout, int64_t n_max,
-    const unsigned long long *n_dev, int shift, int nblocks, const uint32_t *__restrict__ offs) {
-    __shared__ uint32_t cnt[kRsBins * kRsThreads];
-    __shared__ uint32_t warp_sums[kRsThreads / 32];
-    const int64_t n = count_of(n_max, n_dev);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t base = (int64_t)blockIdx.x * kRsTile + (int64_t)tid * kRsItems;
-    uint64_t k[kRsItems];
-    uint32_t val[kRsItems];
-    int d[kRsItems];
-    uint32_t c[kRsBins];
-#pragma unroll
-    for (int b = 0; b < kRsBins; ++b) c[b] = 0u;
-#pragma unroll
-    for (int i = 0; i < kRsItems; ++i) {
-        const int64_t idx = base + i;
-        if (idx < n) {
-            k[i] = kin[idx];
-            val[i] = vin[idx];
-            d[i] = (int)((k[i] >> shift) & (kRsBins - 1));
-#pragma unroll
-            for (int b = 0; b < kRsBins; ++b) c[b] += (d[i] == b);
-        } else {
-            d[i] = -1;
-        }
-    }
-    // digit-major layout [digit][thread]; scan it flat, then subtract the
-    // digit's start to get the count of that digit in earlier threads
-#pragma unroll
-    for (int b = 0; b < kRsBins; ++b) cnt[b * kRsThreads + tid] = c[b];
-    __syncthreads();
-    // each thread scans 16 consecutive entries of the flat array
-    uint32_t loc[kRsBins], sum = 0;
-#pragma unroll
-    for (int j = 0; j < kRsBins; ++j) {
-        loc[j] = sum;
-        sum += cnt[tid * kRsBins + j];
-    }
-    uint32_t incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) warp_sums[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t s = lane < kRsThreads / 32 ? warp_sums[lane] : 0u;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
-        }
-        if (lane < kRsThreads / 32) warp_sums[lane] = s;
-    }
-    __syncthreads();
-    const uint32_t excl = incl - sum + (warp > 0 ? warp_sums[warp - 1] : 0u);
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < kRsBins; ++j) cnt[tid * kRsBins + j] = excl + loc[j];
-    __syncthreads();
-    uint32_t run[kRsBins];
-#pragma unroll
-    for (int b = 0; b < kRsBins; ++b) {
-        const uint32_t start = cnt[b * kRsThreads];  // flat prefix at (digit b, thread 0)
-        run[b] = offs[(int64_t)b * nblocks + blockIdx.x] + (cnt[b * kRsThreads + tid] - start);
-    }
-#pragma unroll
-    for (int i = 0; i < kRsItems; ++i) {
-        if (d[i] < 0) continue;
-        uint32_t pos = 0;
-#pragma unroll
-        for (int b = 0; b < kRsBins; ++b)
-            if (d[i] == b) pos = run[b]++;
-        kout[pos] = k[i];
-        vout[pos] = val[i];
-    }
-}
 
 // Keys of the depth ranking: view depth bits (positive floats order as
 // unsigned integers) in the high word, invisible Gaussians last.
@@ -319,30 +160,6 @@ __global__ void __launch_bounds__(64) k_raster_sorted(RenderArgs args, const uin
 }
 
 }  // namespace
-
-// Sorts (key, value) pairs by bits [begin_bit, end_bit) of the key (stable
-// LSD, 4-bit digits).  n_max bounds the element count and sizes the grids;
-// n_dev (nullable) holds the actual count on the device.  The result is in
-// *k / *v (pointers swapped with the temporaries as needed).
-cudaError_t radix_sort(uint64_t **k, uint32_t **v, uint64_t **kt, uint32_t **vt, int64_t n_max,
-                       const unsigned long long *n_dev, int begin_bit, int end_bit,
-                       uint32_t *hist, cudaStream_t stream) {
-    if (n_max <= 1) return cudaSuccess;
-    const int nblocks = (int)((n_max + kRsTile - 1) / kRsTile);
-    for (int shift = begin_bit; shift < end_bit; shift += 4) {
-        k_rs_hist<<<nblocks, kRsThreads, 0, stream>>>(*k, n_max, n_dev, shift, nblocks, hist);
-        k_rs_scan<<<1, 1024, 0, stream>>>(hist, (int64_t)kRsBins * nblocks);
-        k_rs_scatter<<<nblocks, kRsThreads, 0, stream>>>(*k, *v, *kt, *vt, n_max, n_dev, shift,
-                                                          nblocks, hist);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        std::swap(*k, *kt);
-        std::swap(*v, *vt);
-    }
-    return cudaSuccess;
-}
-
-int64_t sorted_hist_entries(int64_t n_max) { return kRsBins * ((n_max + kRsTile - 1) / kRsTile); }
 
 size_t sorted_temp_bytes(int64_t n, int64_t capacity, int T) {
     size_t a = 0, b = 0;
