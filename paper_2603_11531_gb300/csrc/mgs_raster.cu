@@ -28,7 +28,9 @@
 // a partial product of at most 2^-12 for each of its pixels, T <= 2^-48, so
 // 1 - T is 1 in FP32 and T c_bg is below 2^-40 for |c_bg| <= 256 (a larger
 // background keeps the updates, and so does the aux output, which returns T).
-// The frozen value stays an upper bound of T.
+// The frozen value stays an upper bound of T.  The tensor-core sums, whose lists are
+// the longer ones, stop at partial products of 2^-8 and |c_bg| <= 4: T <= 2^-32 and
+// T c_bg <= 2^-30, below half a unit in the last place of any colour above 2^-6.
 #include "mgs_internal.cuh"
 
 namespace mgs {
@@ -38,6 +40,8 @@ constexpr int kThreads = 128;
 constexpr int kWarps = kThreads / 32;
 constexpr float kFrozenT = 0.000244140625f;   // 2^-12
 constexpr float kMaxFrozenBg = 256.0f;
+constexpr float kFrozenTcT = 0.00390625f;     // 2^-8, tensor-core sums
+constexpr float kMaxFrozenTcBg = 4.0f;
 constexpr int kFreezeEvery = 128;             // list entries between two checks
 constexpr float kLogClamp = -0.014499569695115089f;   // log2(0.99)
 
@@ -135,13 +139,13 @@ __device__ __forceinline__ void accumulate(const ulonglong2 (*wb)[kRingF], int k
     }
 }
 
-// Does every lane hold partial products of at most kFrozenT?
-__device__ __forceinline__ bool all_frozen(float m) {
-    return __all_sync(0xffffffffu, m <= kFrozenT);
+// Does every lane hold partial products of at most `bound`?
+__device__ __forceinline__ bool all_frozen(float m, float bound) {
+    return __all_sync(0xffffffffu, m <= bound);
 }
 
-__device__ __forceinline__ bool may_freeze(const RenderArgs &args) {
-    return fmaxf(fmaxf(fabsf(args.bg[0]), fabsf(args.bg[1])), fabsf(args.bg[2])) <= kMaxFrozenBg;
+__device__ __forceinline__ bool may_freeze(const RenderArgs &args, float max_bg) {
+    return fmaxf(fmaxf(fabsf(args.bg[0]), fabsf(args.bg[1])), fabsf(args.bg[2])) <= max_bg;
 }
 
 // Writes one pixel's outputs from its sums.
@@ -253,7 +257,7 @@ __device__ __forceinline__ void raster_tile(const RenderArgs &args, int tile, Fm
     int head = 0, count = 0;   // queued candidates: ring slots [head, head + count) mod kRingF
     int clamp_left = 0;        // queued candidates up to the last whose opacity exceeds 0.99
     bool live = true;          // T is still updated
-    const bool freeze = !kAux && may_freeze(args);
+    const bool freeze = !kAux && may_freeze(args, kMaxFrozenBg);
     auto group = [&]() {
         const int k = head + t;
         if (live) {
@@ -314,7 +318,7 @@ __device__ __forceinline__ void raster_tile(const RenderArgs &args, int tile, Fm
                 m = fmaxf(m, fmaxf(x, y));
                 if (!(x <= 1.0f && y <= 1.0f)) m = 1.0f;   // NaN: keep updating
             }
-            live = !all_frozen(m);
+            live = !all_frozen(m, kFrozenT);
         }
         __syncwarp();
     }
@@ -375,6 +379,15 @@ __device__ __forceinline__ void raster_tile(const RenderArgs &args, int tile, Fm
 // when the frame's largest weight would overflow FP16 (the scale cancels in
 // A / B and is divided out here).  T stays in FP32 FMAs.  Tiles listing a Gaussian
 // outside that scale's range (kTileWide) are rasterised by the FMA tile code.
+//
+// Bound: instruction issue (83 % of the slots used; a packed FP32x2 operation takes
+// two), so the time follows the instructions per pixel: without T's two FMAs where T
+// is frozen, and with the weight fragment read by one ldmatrix instead of two 16-bit
+// loads and a merge, 600k Gaussians at 1600x1063 take 0.814 ms (0.863 before; either
+// change alone 0.841 and 0.866), depth of 300k at 1280x720 0.381 ms (0.388).  Lists
+// too short to freeze pay about 1 us per launch for the choice (50k at 640x480: 34.7
+// against 33.8 us).  Two lanes per record instead of one (cp.async into shared memory)
+// saves L1 tag lookups but waits longer: 0.876 ms.
 constexpr int kChunk = 8;        // candidates per MMA (K)
 constexpr int kRing = 64;        // candidate slots per warp: eight chunks (a power of two)
 
@@ -405,9 +418,10 @@ __device__ __forceinline__ void mma_k8(float (&d)[4], uint32_t a0, uint32_t a1, 
 // One chunk of 8 candidates starting at ring slot c0 (a multiple of 8): the
 // lane's entries 2t, 2t + 1 at its eight pixels (same FP32 sequence as
 // accumulate()), T updated, alphas packed to FP16 and summed by four MMAs.
+// kLive: T is updated (two of about 17 issue slots per pixel).
 // kDepth: also AD[j] += (a, b) * (w d of the two entries), the FP32 numerator
 // of the depth image (Eq. 5), kept as two partial sums per pixel.
-template <bool kCount, bool kClamp, bool kDepth = false>
+template <bool kCount, bool kClamp, bool kDepth, bool kLive>
 __device__ __forceinline__ void tc_chunk(const float4 (*geo)[kRing / 2], const uint4 *wt,
                                          int c0, int g, int t, const f2 (&pxc)[8], f2 pyc,
                                          f2 kq2, float (&T)[8], float (&D)[4][4], int (&cnt)[8],
@@ -441,13 +455,17 @@ __device__ __forceinline__ void tc_chunk(const float4 (*geo)[kRing / 2], const u
         aa = qa <= 9.0f ? aa : 0.0f;
         ab = qb <= 9.0f ? ab : 0.0f;
         if (kCount) cnt[j] += (qa <= 9.0f) + (qb <= 9.0f);
-        T[j] = fmaf(-aa, T[j], T[j]);
-        T[j] = fmaf(-ab, T[j], T[j]);
+        if constexpr (kLive) {
+            T[j] = fmaf(-aa, T[j], T[j]);
+            T[j] = fmaf(-ab, T[j], T[j]);
+        }
         if constexpr (kDepth) AD[j] = fma2(pk(aa, ab), wdp, AD[j]);
         a[j] = h2bits(aa, ab);            // k = 2t (low half), 2t + 1
     }
-    const unsigned short *wa = reinterpret_cast<const unsigned short *>(wt + c0 + 2 * t);
-    const uint32_t b0 = (uint32_t)wa[g] | ((uint32_t)wa[8 + g] << 16);   // column g, k = 2t, 2t + 1
+    uint32_t b0;   // column g, k = 2t, 2t + 1: the chunk's weights transposed
+    asm volatile("ldmatrix.sync.aligned.m8n8.x1.trans.shared.b16 {%0}, [%1];"
+                 : "=r"(b0)
+                 : "r"((uint32_t)__cvta_generic_to_shared(wt + c0 + (threadIdx.x & 7))));
 #pragma unroll
     for (int i = 0; i < 4; ++i) mma_k8(D[i], a[2 * i], a[2 * i + 1], b0);   // pixels 2i, 2i + 1
 }
@@ -494,6 +512,22 @@ __device__ __forceinline__ void raster_tile_tc(const RenderArgs &args, int tile,
 
     int head = 0, count = 0;          // unprocessed candidates: ring slots [head, head + count)
     uint64_t clamp_mask = 0;          // ring slots whose opacity exceeds 0.99
+    const bool freeze = !kAux && may_freeze(args, kMaxFrozenTcBg);
+    bool live = true;                 // T is still updated
+    auto chunk = [&]() {
+        const bool clamp = ((clamp_mask >> head) & 0xFFull) != 0;
+        if (kAux || live) {
+            if (clamp)
+                tc_chunk<kCount, true, kDepth, true>(geo, wt, head, g, t, pxc, pyc, kq2, T, D, cnt, wd, AD);
+            else
+                tc_chunk<kCount, false, kDepth, true>(geo, wt, head, g, t, pxc, pyc, kq2, T, D, cnt, wd, AD);
+        } else {
+            if (clamp)
+                tc_chunk<kCount, true, kDepth, false>(geo, wt, head, g, t, pxc, pyc, kq2, T, D, cnt, wd, AD);
+            else
+                tc_chunk<kCount, false, kDepth, false>(geo, wt, head, g, t, pxc, pyc, kq2, T, D, cnt, wd, AD);
+        }
+    };
     // prefetch of the next batch: everything the block test and staging need
     float4 a_n = make_float4(0.f, 0.f, 0.f, 0.f);
     float2 b_n = make_float2(0.f, 0.f);
@@ -557,13 +591,16 @@ __device__ __forceinline__ void raster_tile_tc(const RenderArgs &args, int tile,
         __syncwarp();
         count += __popc(bal);
         while (count >= kChunk) {
-            if ((clamp_mask >> head) & 0xFFull)
-                tc_chunk<kCount, true, kDepth>(geo, wt, head, g, t, pxc, pyc, kq2, T, D, cnt, wd, AD);
-            else
-                tc_chunk<kCount, false, kDepth>(geo, wt, head, g, t, pxc, pyc, kq2, T, D, cnt, wd, AD);
+            chunk();
             clamp_mask &= ~(0xFFull << head);
             head = (head + kChunk) & (kRing - 1);
             count -= kChunk;
+        }
+        if (freeze && live && ((base - start) & (kFreezeEvery - 1)) == kFreezeEvery - 32) {
+            float m = T[0];
+#pragma unroll
+            for (int k = 1; k < 8; ++k) m = T[k] <= m ? m : T[k];   // NaN: keep updating
+            live = !all_frozen(m, kFrozenTcT);
         }
         __syncwarp();
     }
@@ -585,10 +622,7 @@ __device__ __forceinline__ void raster_tile_tc(const RenderArgs &args, int tile,
             if constexpr (kDepth) reinterpret_cast<float *>(&wd[pos >> 1])[o] = 0.0f;
         }
         __syncwarp();
-        if ((clamp_mask >> head) & 0xFFull)
-            tc_chunk<kCount, true, kDepth>(geo, wt, head, g, t, pxc, pyc, kq2, T, D, cnt, wd, AD);
-        else
-            tc_chunk<kCount, false, kDepth>(geo, wt, head, g, t, pxc, pyc, kq2, T, D, cnt, wd, AD);
+        chunk();
     }
 
     // Quad reduction: columns c and c + 4 (lanes t, t ^ 2), then swap halves
