@@ -245,7 +245,8 @@ mgs_status render_impl(mgs_workspace w, mgs_scene s, const mgs_camera *cam,
                        const mgs_render_opts *opts, float *out_rgb, float *out_aux,
                        int32_t *out_count, cudaStream_t stream,
                        const BackwardIO *bwd = nullptr, RenderArgs *prep = nullptr,
-                       float *out_depth = nullptr, bool args_only = false) {
+                       float *out_depth = nullptr, bool args_only = false,
+                       bool grouped = false) {
     if (!w || !s) return fail(MGS_ERR_INVALID_ARG, "workspace or scene is NULL");
     if (w->ctx != s->ctx) return fail(MGS_ERR_INVALID_ARG, "scene and workspace belong to different contexts");
     mgs_status st = check_camera(cam);
@@ -323,7 +324,7 @@ mgs_status render_impl(mgs_workspace w, mgs_scene s, const mgs_camera *cam,
         return cuda_fail(e, "preprocess launch");
     if (w->timing) cudaEventRecord(ev[1], stream);
     if ((e = launch_binning(a, w->ctx->sm_count, w->bases, stream,
-                            w->timing ? &ev[2] : nullptr)) != cudaSuccess)
+                            w->timing ? &ev[2] : nullptr, grouped)) != cudaSuccess)
         return cuda_fail(e, "binning launch");
     if (w->timing) cudaEventRecord(ev[5], stream);
     if (opts->flags & MGS_FLAG_SORTED) {
@@ -408,9 +409,9 @@ mgs_status mgs::validate_camera(const mgs_camera *c) { return check_camera(c); }
 
 mgs_status mgs::prepare_view(mgs_workspace w, mgs_scene s, const mgs_camera *cam,
                              const mgs_render_opts *opts, float *out_rgb, cudaStream_t stream,
-                             RenderArgs *args_out, bool args_only) {
+                             RenderArgs *args_out, bool args_only, bool grouped) {
     mgs_status st = render_impl(w, s, cam, opts, out_rgb, nullptr, nullptr, stream, nullptr,
-                                args_out, nullptr, args_only);
+                                args_out, nullptr, args_only, grouped);
     if (st == MGS_OK) args_out->out_rgb = out_rgb;
     return st;
 }

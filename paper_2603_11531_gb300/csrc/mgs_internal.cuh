@@ -306,10 +306,11 @@ cudaError_t launch_preprocess(const RenderArgs &a, int sm_count, cudaStream_t st
 // tile counts and writes the group costs).  `scratch` has bin_scratch_words(n,
 // T, sm_count) 32-bit words: the per-CTA tile bases, then the scan of the
 // 32-Gaussian groups' costs and (at bin_group_cost()) the costs.
+// grouped: other views are binned at the same time (a server's group).
 // marks (nullable): three events recorded on `stream` after the plan scan,
 // after the count and after the tile scan.
 cudaError_t launch_binning(const RenderArgs &a, int sm_count, uint32_t *scratch, cudaStream_t stream,
-                           const cudaEvent_t *marks = nullptr);
+                           const cudaEvent_t *marks = nullptr, bool grouped = false);
 int bin_ctas(int64_t n, int sm_count);
 uint32_t *bin_group_cost(uint32_t *scratch, int64_t n, int64_t T, int sm_count);
 __host__ __device__ constexpr int64_t bin_scratch_words_for(int64_t ctas, int64_t T, int64_t n) {
@@ -335,9 +336,10 @@ mgs_status validate_camera(const mgs_camera *c);
 // no allocation if the workspace is large enough); *args_out receives the
 // arguments the rasteriser needs.  Stream-ordered, capturable.  args_only:
 // check the arguments, size the workspace and fill *args_out, launch nothing.
+// grouped: see launch_binning.
 mgs_status prepare_view(mgs_workspace w, mgs_scene s, const mgs_camera *cam,
                         const mgs_render_opts *opts, float *out_rgb, cudaStream_t stream,
-                        RenderArgs *args_out, bool args_only = false);
+                        RenderArgs *args_out, bool args_only = false, bool grouped = false);
 // Changes whenever one of the workspace's scratch buffers is reallocated
 // (launches captured before then address freed memory).
 uint64_t workspace_generation(mgs_workspace w);

@@ -187,7 +187,8 @@ mgs_status launch_view(mgs_server_s *S, Slot &sl, Request &rq, bool raster) {
     // Stream-ordered preparation; sets sl.args (needed for the batched raster
     // and the status read-back) and grows the workspace if it must.
     auto direct = [&]() -> mgs_status {
-        mgs_status st = prepare_view(sl.ws, rq.scene, &rq.cam, &rq.opts, rq.out, sl.stream, &sl.args);
+        mgs_status st = prepare_view(sl.ws, rq.scene, &rq.cam, &rq.opts, rq.out, sl.stream, &sl.args,
+                                     false, !raster);
         if (st == MGS_OK && raster && launch_raster(sl.args, sl.stream) != cudaSuccess)
             st = MGS_ERR_CUDA;
         return st;
@@ -232,7 +233,7 @@ mgs_status launch_view(mgs_server_s *S, Slot &sl, Request &rq, bool raster) {
     mgs_status st = MGS_ERR_CUDA;
     cudaError_t e = cudaStreamBeginCapture(sl.stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        st = prepare_view(sl.ws, rq.scene, &rq.cam, &rq.opts, rq.out, sl.stream, &a);
+        st = prepare_view(sl.ws, rq.scene, &rq.cam, &rq.opts, rq.out, sl.stream, &a, false, !raster);
         if (st == MGS_OK && raster && launch_raster(a, sl.stream) != cudaSuccess) st = MGS_ERR_CUDA;
         e = cudaStreamEndCapture(sl.stream, &g);
     }
