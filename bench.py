@@ -283,10 +283,10 @@ def cpu_baseline_frame(pose: int = 0):
 
 
 # Kernels of this library one FP16 render launches: k_preprocess,
-# k_bin_plan, k_bin_count, k_scan_order, k_bin_scatter and
-# k_raster_tc, once each.  The ncu launch list of a bench run shows the same
+# k_bin_count, k_scan_order, k_bin_scatter and k_raster_tc, once
+# each.  The ncu launch list of a bench run shows the same
 # set per frame.
-KERNELS_PER_FRAME = 6
+KERNELS_PER_FRAME = 5
 
 
 def run_reference(args):

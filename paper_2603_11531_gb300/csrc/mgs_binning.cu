@@ -4,12 +4,12 @@
 // (Sec. 2, Eq. 1 discussion; Sec. 3.1).  The lists built here are keyed by
 // tile only -- a counting sort by tile:
 //
-//   0. k_bin_plan: the exclusive scan of the groups' plan costs (a group is 32
-//      consecutive Gaussians; preprocessing has summed the costs of its
-//      rectangle rows, kRowCost plus the row's width in tiles each) plus a
-//      fixed visit charge.  Every warp of the binning grid (at most one
-//      512-thread CTA per SM) takes an equal contiguous share of that cost
-//      numbering, cut at row boundaries.
+//   0. the work plan, at the start of k_bin_count: every warp of the binning
+//      grid (at most one 512-thread CTA per SM) takes an equal contiguous share
+//      of the cost numbering of all rectangle rows, cut at row boundaries.
+//      Preprocessing has summed the rows' costs (kRowCost plus the row's width
+//      in tiles) per group of 32 consecutive Gaussians; each group adds a fixed
+//      visit charge.
 //   1. k_bin_count: each warp resolves its rows, 32 at a time (one per lane):
 //      the tiles of a rectangle row that pass the FP32 tile test form one
 //      interval (row_tiles), which is added to a per-CTA shared-memory
@@ -425,65 +425,75 @@ __device__ __forceinline__ void warp_rows(const GroupLoad &L, int64_t g0, int ca
     }
 }
 
-// Largest group g with cexcl[g] <= c (c < cexcl[groups]); the warp probes 32
-// entries at a time (three dependent loads for 18,750 groups instead of the
-// fifteen of a binary search, about 4 us of the count and of the scatter).
-__device__ __forceinline__ int64_t find_group(const unsigned long long *__restrict__ cexcl,
-                                              int64_t groups, unsigned long long c) {
-    const int lane = threadIdx.x & 31;
-    int64_t lo = 0, hi = groups;   // cexcl[lo] <= c < cexcl[hi]
-    while (hi - lo > 1) {
-        const int64_t step = (hi - lo + 31) / 32;
-        const int64_t p = lo + step * (lane + 1);
-        const unsigned le = __ballot_sync(0xffffffffu, p < hi && cexcl[p] <= c);
-        lo += step * __popc(le);
-        if (lo + step < hi) hi = lo + step;
+// A warp's share of the cost numbering: len costs from c0 on.  The group it starts
+// in begins `before` costs earlier (less than one group's cost).
+struct Share {
+    unsigned long long c0;
+    long long len;
+    uint32_t before;
+    int group;
+};
+
+// What k_bin_count hands to k_bin_scatter: plan[0] is the total cost C, plan[1 + w]
+// the {group, before} of warp w.  At most one share per group, so that the plan
+// fits its scratch of groups + 1 entries.
+__device__ __forceinline__ Share share_of(unsigned long long C, int groups) {
+    const unsigned long long all = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+    const unsigned long long W = all < (unsigned long long)groups ? all : (unsigned long long)groups;
+    const unsigned long long w = (unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    Share sh{0ull, 0, 0u, 0};
+    if (w < W) {
+        sh.c0 = C * w / W;
+        sh.len = (long long)(C * (w + 1) / W - sh.c0);
     }
-    return lo;
+    return sh;
 }
 
-// Calls f(active, item) for the rows of this warp's share of the work plan:
-// group g occupies costs [cexcl[g], cexcl[g + 1]), its visit charge first and
-// then its row costs; warp w of W takes costs [C w / W, C (w + 1) / W) of the
-// total C, and a row belongs to the share holding its start cost.  The plan
-// entries are read 32 at a time and groups without rows (all Gaussians
-// culled) are skipped without loading them; each group with rows is loaded
-// while the previous one is processed.
+// Calls f(active, item) for the rows of this warp's share of the work plan: a
+// group's visit charge comes first and then its row costs, and a row belongs to
+// the share holding its start cost.  The groups' costs are read 32 at a time
+// (the next 32 ahead) and groups without rows (all Gaussians culled) are skipped
+// without loading them; each group with rows is loaded while the previous one is
+// processed.
 template <class F>
 __device__ __forceinline__ void warp_share_rows(const uint2 *__restrict__ rect,
                                                 const ProjRec *__restrict__ rec, int64_t n,
-                                                const unsigned long long *__restrict__ cexcl,
-                                                int64_t groups, RowSlot *q, F &&f) {
-    if (groups == 0) return;
+                                                const uint32_t *__restrict__ cost, int groups,
+                                                const Share &sh, RowSlot *q, F &&f) {
     const int lane = threadIdx.x & 31;
     int qh = 0, qn = 0;   // queued rows: slots [qh, qh + qn) mod kQueue
-    const unsigned long long C = cexcl[groups];
-    const unsigned long long W = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-    const unsigned long long w = (unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const unsigned long long c0 = C * w / W, c1 = C * (w + 1) / W;
-    if (c0 >= c1) return;
-    for (int64_t gb = find_group(cexcl, groups, c0); gb < groups; gb += 32) {
-        const int64_t gl = gb + lane;
-        const unsigned long long e0l = gl < groups ? cexcl[gl] : C;
-        const unsigned long long e1l = gl < groups ? cexcl[gl + 1] : C;
-        // groups of this chunk with rows whose row costs meet [c0, c1)
-        unsigned m = __ballot_sync(0xffffffffu, gl < groups && e1l - e0l > (unsigned long long)kGroupCost &&
-                                                    e1l > c0 && e0l + kGroupCost < c1);
-        const bool done = __ballot_sync(0xffffffffu, gl >= groups || e1l >= c1) != 0u;
+    if (sh.len <= 0) return;
+    long long e = -(long long)sh.before;   // cost at which group gb starts, from c0 on
+    uint32_t v_n = sh.group + lane < groups ? cost[sh.group + lane] : 0u;
+    for (int gb = sh.group; gb < groups; gb += 32) {
+        const int gl = gb + lane;
+        const long long v = gl < groups ? (long long)v_n + kGroupCost : 0;
+        v_n = gl + 32 < groups ? cost[gl + 32] : 0u;
+        long long e1l = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long y = __shfl_up_sync(0xffffffffu, e1l, o);
+            if (lane >= o) e1l += y;
+        }
+        e1l += e;
+        const long long e0l = e1l - v;
+        e = __shfl_sync(0xffffffffu, e1l, 31);
+        // groups of this chunk with rows whose row costs meet the share
+        unsigned m = __ballot_sync(0xffffffffu, v > kGroupCost && e1l > 0 && e0l + kGroupCost < sh.len);
+        const bool done = __ballot_sync(0xffffffffu, gl >= groups || e1l >= sh.len) != 0u;
         if (m) {
             int j = __ffs(m) - 1;
             m &= m - 1;
-            GroupLoad cur = load_group(rect, rec, n, (gb + j) * 32);
+            GroupLoad cur = load_group(rect, rec, n, (int64_t)(gb + j) * 32);
             for (;;) {
                 const int jn = m ? __ffs(m) - 1 : -1;
                 GroupLoad nxt{};
-                if (jn >= 0) nxt = load_group(rect, rec, n, (gb + jn) * 32);   // in flight meanwhile
-                const unsigned long long e0 = __shfl_sync(0xffffffffu, e0l, j);
-                const unsigned long long e1 = __shfl_sync(0xffffffffu, e1l, j);
-                const long long nc = (long long)(e1 - e0) - kGroupCost;    // row costs of the group
-                const long long ca = max(0ll, (long long)(c0 > e0 ? c0 - e0 : 0ull) - kGroupCost);
-                const long long cb = min(nc, (long long)(c1 - e0) - kGroupCost);
-                if (ca < cb) warp_rows(cur, (gb + j) * 32, (int)ca, (int)cb, q, qh, qn, f);
+                if (jn >= 0) nxt = load_group(rect, rec, n, (int64_t)(gb + jn) * 32);   // in flight meanwhile
+                const long long e0 = __shfl_sync(0xffffffffu, e0l, j) + kGroupCost;   // row costs start
+                const long long nc = __shfl_sync(0xffffffffu, e1l, j) - e0;
+                const long long ca = max(0ll, -e0);
+                const long long cb = min(nc, sh.len - e0);
+                if (ca < cb) warp_rows(cur, (int64_t)(gb + j) * 32, (int)ca, (int)cb, q, qh, qn, f);
                 if (jn < 0) break;
                 j = jn;
                 m &= m - 1;
@@ -495,62 +505,124 @@ __device__ __forceinline__ void warp_share_rows(const uint2 *__restrict__ rect,
     if (qn > 0) run_rows(q, qh, qn, f);
 }
 
-// Exclusive scan of the group costs (plus kGroupCost) into cexcl[0..groups]
-// (64-bit), by one block, kPlanSeg groups at a time staged in shared memory
-// so that global loads and stores stay coalesced.
-constexpr int kPlanSeg = 16384;   // 64-bit costs per pass
-// Shared-memory slot of entry i: one pad word every 16 entries, so that
-// threads scanning runs of 16 consecutive entries hit different banks.
-__device__ __forceinline__ int plan_slot(int i) { return i + (i >> 4); }
-constexpr int kPlanSlots = kPlanSeg + kPlanSeg / 16;
-__global__ void __launch_bounds__(kScanThreads) k_bin_plan(const uint32_t *__restrict__ grp,
-                                                           int64_t groups,
-                                                           unsigned long long *__restrict__ cexcl) {
-    grid_wait();
-    extern __shared__ unsigned long long seg[];
-    __shared__ unsigned long long warp_sums[kScanThreads / 32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    unsigned long long carry = 0;   // identical in every thread
-    for (int64_t s0 = 0; s0 < groups; s0 += kPlanSeg) {
-        const int m = (int)(groups - s0 < kPlanSeg ? groups - s0 : kPlanSeg);
-        for (int i = tid; i < m; i += kScanThreads)
-            seg[plan_slot(i)] = (unsigned long long)grp[s0 + i] + kGroupCost;
-        __syncthreads();
-        const int per = (m + kScanThreads - 1) / kScanThreads;
-        const int lo = min(tid * per, m), hi = min(lo + per, m);
-        unsigned long long local = 0;
-        for (int i = lo; i < hi; ++i) local += seg[plan_slot(i)];
-        unsigned long long incl = local;
+// The CTA's shares.  Every CTA sums all group costs by chunks (4 bytes per 32
+// Gaussians, from L2), scans the chunks' sums in shared memory, and each warp
+// looks its start up: chunk by the scan, then group inside the chunk.  Bound: the
+// latency of these dependent loads; in each CTA it costs 1 us (50k Gaussians), 5 us
+// (600k) or 65 us (6M) of the count.  One CTA that scans for all (7, 14 and 85 us) is
+// a launch more and leaves every warp three dependent searches in the count and in
+// the scatter: 50k at 640x480 65.2 us a frame with it, 63.4 without; depth of 300k
+// 479.6 and 474.5 us; 600k at 1600x1063 1039 and 1034.5 us.
+constexpr int kPlanChunk = 128;      // groups per chunk, doubled until they fit
+constexpr int kPlanChunks = 2048;
+struct PlanSmem {
+    unsigned long long pre[kPlanChunks + 1];   // costs before each chunk, total last
+    unsigned long long warp_sums[kBinThreads / 32];
+};
+static_assert(kPlanChunks == 4 * kBinThreads, "four chunks per thread in the scan");
+
+__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+__device__ __forceinline__ Share plan_shares(const uint32_t *__restrict__ cost, int groups,
+                                             PlanSmem &sm, unsigned long long *__restrict__ plan) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    int size = kPlanChunk;
+    while ((int64_t)size * kPlanChunks < groups) size *= 2;
+    const int chunks = (groups - 1) / size + 1;
+#pragma unroll 4
+    for (int c = warp; c < chunks; c += kBinThreads / 32) {
+        unsigned long long sum = 0;
+        const int end = (int)min((int64_t)groups, (int64_t)(c + 1) * size);
+        for (int g = c * size + lane; g < end; g += kPlanChunk) {
+            uint32_t v[kPlanChunk / 32];
+#pragma unroll
+            for (int k = 0; k < kPlanChunk / 32; ++k) v[k] = g + 32 * k < end ? cost[g + 32 * k] : 0u;
+#pragma unroll
+            for (int k = 0; k < kPlanChunk / 32; ++k)
+                sum += (unsigned long long)v[k] + (g + 32 * k < end ? kGroupCost : 0);
         }
-        if (lane == 31) warp_sums[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            unsigned long long t = warp_sums[lane];
+        sum = warp_sum(sum);
+        if (lane == 0) sm.pre[c] = sum;
+    }
+    __syncthreads();
+    // exclusive scan of the chunks
+    unsigned long long v[4], local = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        v[k] = 4 * tid + k < chunks ? sm.pre[4 * tid + k] : 0ull;
+        local += v[k];
+    }
+    unsigned long long incl = local;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) sm.warp_sums[warp] = incl;
+    __syncthreads();
+    unsigned long long run = incl - local, C = 0;
+    for (int w = 0; w < kBinThreads / 32; ++w) {
+        if (w < warp) run += sm.warp_sums[w];
+        C += sm.warp_sums[w];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (4 * tid + k < chunks) sm.pre[4 * tid + k] = run;
+        run += v[k];
+    }
+    if (tid == 0) sm.pre[chunks] = C;
+    __syncthreads();
+
+    Share sh = share_of(C, groups);
+    if (blockIdx.x == 0 && tid == 0) plan[0] = C;
+    if (sh.len > 0) {
+        int lo = 0, hi = chunks;   // pre[lo] <= c0 < pre[hi]
+        while (hi - lo > 1) {
+            const int step = (hi - lo + 31) / 32;
+            const int p = lo + step * (lane + 1);
+            const unsigned le = __ballot_sync(0xffffffffu, p < hi && sm.pre[p] <= sh.c0);
+            lo += step * __popc(le);
+            if (lo + step < hi) hi = lo + step;
+        }
+        unsigned long long e = sm.pre[lo];
+        // the group inside the chunk: it exists, c0 < pre[lo + 1]
+        for (int g = lo * size; g < groups; g += 32) {
+            const unsigned long long c = g + lane < groups ? (unsigned long long)cost[g + lane] + kGroupCost : 0ull;
+            unsigned long long end = c;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long y = __shfl_up_sync(0xffffffffu, t, o);
-                if (lane >= o) t += y;
+                const unsigned long long y = __shfl_up_sync(0xffffffffu, end, o);
+                if (lane >= o) end += y;
             }
-            warp_sums[lane] = t;
+            const unsigned long long total = __shfl_sync(0xffffffffu, end, 31);
+            if (e + total > sh.c0) {
+                const int k = __popc(__ballot_sync(0xffffffffu, e + end <= sh.c0));   // lanes before it
+                sh.group = g + k;
+                sh.before = (uint32_t)(sh.c0 - e - __shfl_sync(0xffffffffu, end - c, k));
+                break;
+            }
+            e += total;
         }
-        __syncthreads();
-        unsigned long long run = carry + (incl - local) + (warp > 0 ? warp_sums[warp - 1] : 0ull);
-        for (int i = lo; i < hi; ++i) {
-            const unsigned long long v = seg[plan_slot(i)];
-            seg[plan_slot(i)] = run;
-            run += v;
-        }
-        carry += warp_sums[kScanThreads / 32 - 1];
-        __syncthreads();
-        for (int i = tid; i < m; i += kScanThreads) cexcl[s0 + i] = seg[plan_slot(i)];
-        __syncthreads();
+        if (lane == 0)
+            plan[1 + blockIdx.x * (kBinThreads / 32) + warp] =
+                (unsigned long long)sh.group << 32 | sh.before;
     }
-    grid_trigger();
-    if (tid == 0) cexcl[groups] = carry;
+    return sh;
+}
+
+// The same share, as k_bin_count stored it.
+__device__ __forceinline__ Share stored_share(const unsigned long long *__restrict__ plan, int groups) {
+    Share sh = share_of(plan[0], groups);
+    if (sh.len > 0) {
+        const unsigned long long p = plan[1 + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)];
+        sh.group = (int)(p >> 32);
+        sh.before = (uint32_t)p;
+    }
+    return sh;
 }
 
 // Tile rows per shared-memory band: the count's difference array takes
@@ -568,8 +640,9 @@ __host__ __device__ __forceinline__ int band_rows(int tiles_x, int tiles_y) {
 __global__ void __launch_bounds__(kBinThreads, 2) k_bin_count(const uint2 *__restrict__ rect,
                                                            const ProjRec *__restrict__ rec,
                                                            int64_t n, int tiles_x, int tiles_y,
-                                                           const unsigned long long *__restrict__ excl,
-                                                           int64_t groups,
+                                                           const uint32_t *__restrict__ cost,
+                                                           int groups,
+                                                           unsigned long long *__restrict__ plan,
                                                            uint32_t *__restrict__ tile_count,
                                                            uint32_t *__restrict__ bases,
                                                            const DevStatus *__restrict__ status,
@@ -577,7 +650,12 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_bin_count(const uint2 *__res
     grid_wait();
     grid_trigger();   // the dependent (the tile scan) is one CTA
     extern __shared__ int diff_s[];
-    __shared__ RowSlot queue_s[kBinThreads / 32][kQueue];
+    __shared__ union {
+        RowSlot queue[kBinThreads / 32][kQueue];
+        PlanSmem plan;
+    } sm;
+    const Share share = plan_shares(cost, groups, sm.plan, plan);
+    __syncthreads();   // the queues take the plan's place
     const int T = tiles_x * tiles_y;
     const int stride = tiles_x + 1;
     const int brows = band_rows(tiles_x, tiles_y);
@@ -590,7 +668,7 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_bin_count(const uint2 *__res
         if (mark)
             for (int i = threadIdx.x; i < nrows * tiles_x; i += kBinThreads) wide_s[i] = 0;
         __syncthreads();
-        warp_share_rows(rect, rec, n, excl, groups, queue_s[warp], [&](bool active, const RowItem &it) {
+        warp_share_rows(rect, rec, n, cost, groups, share, sm.queue[warp], [&](bool active, const RowItem &it) {
             const int ry = it.ty - ty0;
             if (!active || (unsigned)ry >= (unsigned)nrows) return;
             int *d = diff_s + ry * stride;
@@ -645,7 +723,7 @@ constexpr int kLaneRun = 16;
 
 __global__ void __launch_bounds__(kBinThreads, 2) k_bin_scatter(
     const uint2 *__restrict__ rect, int64_t n, int tiles_x, int tiles_y,
-    const unsigned long long *__restrict__ excl, int64_t groups,
+    const uint32_t *__restrict__ cost, int groups, const unsigned long long *__restrict__ plan,
     const uint32_t *__restrict__ offsets, const uint32_t *__restrict__ bases,
     uint32_t *__restrict__ gids, uint64_t capacity, const DevStatus *__restrict__ status,
     const ProjRec *__restrict__ rec, uint4 *__restrict__ wt16) {
@@ -653,6 +731,7 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_bin_scatter(
     extern __shared__ uint32_t cur_s[];
     __shared__ RowSlot queue_s[kBinThreads / 32][kQueue];
     if (status->last_pairs > capacity) return;  // overflow: lists are not built
+    const Share share = stored_share(plan, groups);
     const int we = (int)((status->wmax_frame_bits >> 23) & 0xFFu) - 127;
     if (wt16 && we >= 14) {   // preprocessing wrote the FP16 weights unscaled; rescale them
         const float scale = __int_as_float((127 + 14 - we) << 23);
@@ -672,7 +751,7 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_bin_scatter(
         for (int i = threadIdx.x; i < bn; i += kBinThreads)
             cur_s[i] = offsets[t0 + i] + bases[(int64_t)blockIdx.x * T + t0 + i];
         __syncthreads();
-        warp_share_rows(rect, rec, n, excl, groups, queue_s[threadIdx.x >> 5], [&](bool active, const RowItem &it) {
+        warp_share_rows(rect, rec, n, cost, groups, share, queue_s[threadIdx.x >> 5], [&](bool active, const RowItem &it) {
             const int ry = it.ty - ty0;
             const bool in = active && (unsigned)ry < (unsigned)nrows;
             int a = 1, b = 0;
@@ -852,7 +931,7 @@ cudaError_t launch_binning(const RenderArgs &a, int sm_count, uint32_t *scratch,
     const int C = grouped ? std::min(CL, std::max(sm_count / 2, 1)) : CL;
     const int64_t groups = (a.n + 31) / 32;
     uint32_t *bases = scratch;
-    unsigned long long *excl =
+    unsigned long long *plan =
         reinterpret_cast<unsigned long long *>(scratch + ((int64_t)CL * T + 1) / 2 * 2);
     const int brows = band_rows(tx, ty);
     const size_t count_smem = ((size_t)brows * (tx + 1) * sizeof(int) + (size_t)brows * tx + 15) / 16 * 16;
@@ -868,17 +947,9 @@ cudaError_t launch_binning(const RenderArgs &a, int sm_count, uint32_t *scratch,
         if ((e = cudaFuncSetAttribute(k_bin_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)(kBand * sizeof(uint32_t)))) != cudaSuccess)
             return e;
-        const int plan_n = (int)(groups < kPlanSeg ? groups : kPlanSeg);
-        const size_t plan_smem = (size_t)(plan_n + plan_n / 16) * sizeof(unsigned long long);
-        if ((e = cudaFuncSetAttribute(k_bin_plan, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(kPlanSlots * sizeof(unsigned long long)))) != cudaSuccess)
-            return e;
-        if ((e = launch_dependent(k_bin_plan, 1, kScanThreads, plan_smem, stream, a.group_cost, groups,
-                                  excl)) != cudaSuccess)
-            return e;
         if (marks && (e = cudaEventRecord(marks[0], stream)) != cudaSuccess) return e;
         if ((e = launch_dependent(k_bin_count, C, kBinThreads, count_smem, stream, a.rect, a.rec, a.n, tx,
-                                  ty, excl, groups, a.tile_count, bases, a.status, tc_raster(a))) !=
+                                  ty, a.group_cost, (int)groups, plan, a.tile_count, bases, a.status, tc_raster(a))) !=
             cudaSuccess)
             return e;
         if (marks && (e = cudaEventRecord(marks[1], stream)) != cudaSuccess) return e;
@@ -891,8 +962,8 @@ cudaError_t launch_binning(const RenderArgs &a, int sm_count, uint32_t *scratch,
         return e;
     if (marks && (e = cudaEventRecord(marks[2], stream)) != cudaSuccess) return e;
     if (a.n == 0) return e;
-    return launch_dependent(k_bin_scatter, C, kBinThreads, scatter_smem, stream, a.rect, a.n, tx, ty, excl,
-                            groups, a.tile_offsets, bases, a.gids, a.capacity, a.status, a.rec,
+    return launch_dependent(k_bin_scatter, C, kBinThreads, scatter_smem, stream, a.rect, a.n, tx, ty,
+                            a.group_cost, (int)groups, plan, a.tile_offsets, bases, a.gids, a.capacity, a.status, a.rec,
                             tc_raster(a) ? a.wt16 : nullptr);
 }
 

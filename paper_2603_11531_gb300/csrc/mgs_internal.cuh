@@ -304,11 +304,11 @@ cudaError_t launch_sorted(const RenderArgs &a, const SortedScratch &s, cudaStrea
 cudaError_t launch_preprocess(const RenderArgs &a, int sm_count, cudaStream_t stream);
 // Per-tile counts, scan and scatter, after launch_preprocess (which clears the
 // tile counts and writes the group costs).  `scratch` has bin_scratch_words(n,
-// T, sm_count) 32-bit words: the per-CTA tile bases, then the scan of the
-// 32-Gaussian groups' costs and (at bin_group_cost()) the costs.
+// T, sm_count) 32-bit words: the per-CTA tile bases, then the work plan and
+// (at bin_group_cost()) the costs of the 32-Gaussian groups.
 // grouped: other views are binned at the same time (a server's group).
-// marks (nullable): three events recorded on `stream` after the plan scan,
-// after the count and after the tile scan.
+// marks (nullable): three events recorded on `stream` before the count,
+// after it and after the tile scan.
 cudaError_t launch_binning(const RenderArgs &a, int sm_count, uint32_t *scratch, cudaStream_t stream,
                            const cudaEvent_t *marks = nullptr, bool grouped = false);
 int bin_ctas(int64_t n, int sm_count);

@@ -182,7 +182,6 @@ __global__ void __launch_bounds__(kWide ? tcw::kThreads : (kTC ? tc::kThreads : 
     constexpr int kStep =
         kWide ? tcw::kThreads : (kTC ? tc::kThreads : kThreads);   // Gaussians per CTA step
     grid_wait();
-    grid_trigger();   // the dependent (the binning plan) is one CTA
     extern __shared__ __align__(128) unsigned char smem_raw[];
     MlpSmem &sm = *reinterpret_cast<MlpSmem *>(smem_raw);
     tc::Smem &tsm = *reinterpret_cast<tc::Smem *>(smem_raw);
