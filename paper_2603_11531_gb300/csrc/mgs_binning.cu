@@ -927,7 +927,9 @@ cudaError_t launch_binning(const RenderArgs &a, int sm_count, uint32_t *scratch,
     // Views prepared side by side fill the chip between them, so each takes at most
     // half as many CTAs: less per-CTA work (clearing and scanning T counts).  A burst of
     // twelve views of 160k Gaussians: 1.087 ms with one CTA per SM and view, 1.078 with
-    // one per two SMs; a quarter and a third of the SMs are slower again.
+    // one per two SMs in a group of views, 1.066 where the lone views of a busy server
+    // do the same; a third and a quarter of the SMs are slower (1.071 and 1.108 where
+    // half took 1.053).
     const int C = grouped ? std::min(CL, std::max(sm_count / 2, 1)) : CL;
     const int64_t groups = (a.n + 31) / 32;
     uint32_t *bases = scratch;

@@ -306,7 +306,7 @@ cudaError_t launch_preprocess(const RenderArgs &a, int sm_count, cudaStream_t st
 // tile counts and writes the group costs).  `scratch` has bin_scratch_words(n,
 // T, sm_count) 32-bit words: the per-CTA tile bases, then the work plan and
 // (at bin_group_cost()) the costs of the 32-Gaussian groups.
-// grouped: other views are binned at the same time (a server's group).
+// grouped: other views are binned or rasterised at the same time (a busy server).
 // marks (nullable): three events recorded on `stream` before the count,
 // after it and after the tile scan.
 cudaError_t launch_binning(const RenderArgs &a, int sm_count, uint32_t *scratch, cudaStream_t stream,

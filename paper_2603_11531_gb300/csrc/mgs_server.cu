@@ -135,12 +135,12 @@ uint64_t cache_key(mgs_scene s, int w, int h) {
     return (reinterpret_cast<uint64_t>(s) * 1000003ull) ^ ((uint64_t)w << 32) ^ (uint64_t)h;
 }
 
-uint64_t graph_key(const Request &rq, bool raster) {
+uint64_t graph_key(const Request &rq, bool raster, bool grouped) {
     uint64_t k = cache_key(rq.scene, rq.cam.width, rq.cam.height);
     k = k * 31ull + (uint64_t)rq.opts.use_mlp;
     k = k * 31ull + (uint64_t)rq.opts.mlp_rgb_residual;
     k = k * 131ull + (uint64_t)rq.opts.flags;
-    return k * 2ull + (raster ? 1ull : 0ull);
+    return k * 4ull + (raster ? 1ull : 0ull) + (grouped ? 2ull : 0ull);
 }
 
 int64_t estimate_bytes(int64_t n, int w, int h, uint64_t pairs, int sm_count) {
@@ -182,19 +182,20 @@ std::vector<cudaGraphNode_t> render_arg_nodes(cudaGraph_t g) {
 
 // The request's work on the slot's stream: preprocessing and binning, and the
 // single-view rasteriser when `raster`.  Through the slot's cached graph for
-// this key when graphs are usable, else by direct launches.
-mgs_status launch_view(mgs_server_s *S, Slot &sl, Request &rq, bool raster) {
+// this key when graphs are usable, else by direct launches.  grouped: see
+// launch_binning.
+mgs_status launch_view(mgs_server_s *S, Slot &sl, Request &rq, bool raster, bool grouped) {
     // Stream-ordered preparation; sets sl.args (needed for the batched raster
     // and the status read-back) and grows the workspace if it must.
     auto direct = [&]() -> mgs_status {
         mgs_status st = prepare_view(sl.ws, rq.scene, &rq.cam, &rq.opts, rq.out, sl.stream, &sl.args,
-                                     false, !raster);
+                                     false, grouped);
         if (st == MGS_OK && raster && launch_raster(sl.args, sl.stream) != cudaSuccess)
             st = MGS_ERR_CUDA;
         return st;
     };
     if (!S->graphs) return direct();
-    const uint64_t key = graph_key(rq, raster);
+    const uint64_t key = graph_key(rq, raster, grouped);
     const uint64_t gen = workspace_generation(sl.ws);
     SlotGraph *hit = nullptr;
     for (SlotGraph &g : sl.graphs)
@@ -233,7 +234,7 @@ mgs_status launch_view(mgs_server_s *S, Slot &sl, Request &rq, bool raster) {
     mgs_status st = MGS_ERR_CUDA;
     cudaError_t e = cudaStreamBeginCapture(sl.stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        st = prepare_view(sl.ws, rq.scene, &rq.cam, &rq.opts, rq.out, sl.stream, &a, false, !raster);
+        st = prepare_view(sl.ws, rq.scene, &rq.cam, &rq.opts, rq.out, sl.stream, &a, false, grouped);
         if (st == MGS_OK && raster && launch_raster(a, sl.stream) != cudaSuccess) st = MGS_ERR_CUDA;
         e = cudaStreamEndCapture(sl.stream, &g);
     }
@@ -418,6 +419,13 @@ void mgs_server_s::run() {
         if (!admitted.empty()) {
             Group &b = groups[bi];
             const bool alone = admitted.size() == 1;
+            // will other views be prepared or rasterised meanwhile?
+            bool grouped = !alone;
+            for (const Group &o : groups) grouped |= o.active;
+            if (!grouped) {
+                std::lock_guard<std::mutex> lk(mu);
+                grouped = !queue.empty();
+            }
             std::vector<int> ok;
             for (int si : admitted) {
                 Slot &sl = slots[si];
@@ -426,7 +434,7 @@ void mgs_server_s::run() {
                     std::lock_guard<std::mutex> lk(mu);
                     rq = &reqs[sl.ticket];
                 }
-                mgs_status st = launch_view(this, sl, *rq, alone);
+                mgs_status st = launch_view(this, sl, *rq, alone, grouped);
                 if (st == MGS_OK && !alone &&
                     cudaEventRecord(sl.prepared, sl.stream) != cudaSuccess)
                     st = MGS_ERR_CUDA;
