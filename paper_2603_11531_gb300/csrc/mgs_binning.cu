@@ -41,9 +41,10 @@ namespace {
 constexpr int kScanThreads = 1024;
 // Count and scatter run one 512-thread CTA per SM at 64 registers a thread:
 // half of the register file, so that the previous frame's rasteriser keeps
-// two CTAs on the SM meanwhile.  Alone, 1024 threads per CTA bin faster (count
-// 0.051 against 0.068 ms on the 600k benchmark view), but frames in flight on
-// several streams render faster this way (971 against 957 FPS).
+// two CTAs on the SM meanwhile.  Alone, more threads bin faster (600k at 1600x1063,
+// 512 / 768 / 1024: count 0.052 / 0.041 / 0.040 ms, scatter 0.121 / 0.116 / 0.116),
+// but frames in flight on several streams render faster this way (1030 / 1024 / 1026
+// FPS, served 870 / 858 / 860 views/s).
 constexpr int kBinThreads = 512;
 constexpr int kBand = 32768;          // words per shared-memory band (128 KB)
 
@@ -899,10 +900,9 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_order(const uint32_t *__r
 // One binning CTA per SM at most: the work plan balances the warps, so a second
 // resident CTA would only add per-CTA tile bases.  Below that, one per 512
 // Gaussians, a group per warp: small scenes are bound by the latency of a warp's
-// walk over its groups (50k frame at 640x480 77 us against 83 us with one CTA
-// per 1024 Gaussians; 4k frame 53 against 60 us), while views served together
-// prefer few CTAs (twelve views of 40k to 160k: 1.08 ms, 1.05 with one per 1024,
-// 1.10 with one per 256).
+// walk over its groups.  One CTA per 256 / 512 / 1024 Gaussians: 4k frame at 256x256
+// 40.4 / 40.4 / 48.2 us, 50k at 640x480 63.7 / 63.5 / 70.8 us, twelve served views of
+// 40k to 160k 1.062 / 1.065 / 1.079 ms.
 int bin_ctas(int64_t n, int sm_count) {
     int64_t c = (n + 511) / 512;
     const int64_t cap = (int64_t)sm_count;
