@@ -30,7 +30,9 @@
  *     reported by mgs_workspace_sync().
  *   - A workspace holds the per-frame scratch (projected Gaussians, tile
  *     lists).  Renders that share a workspace must be ordered on one stream;
- *     concurrent renders need one workspace each.
+ *     concurrent renders need one workspace each.  After mgs_render_backward
+ *     the workspace orders itself: a later call on another stream waits (on
+ *     the device) for the backward pass's kernels.
  */
 #ifndef MOBILEGS_H
 #define MOBILEGS_H

@@ -47,14 +47,6 @@ def _step_scene(renderer, attrs, mlp):
     return mgs_borrow_scene(renderer.ctx, a, params, blob), (a, blob)
 
 
-def _after_last_backward(renderer, stream):
-    """Orders `stream` after the renderer's last backward, which returns before
-    its kernels are done with the renderer's workspace."""
-    last = getattr(renderer, "_backward_done", None)
-    if last is not None and last[0] != stream:
-        stream.wait_event(last[1])
-
-
 class RenderFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, renderer, cam, opts, attrs, *mlp):
@@ -64,7 +56,6 @@ class RenderFn(torch.autograd.Function):
             H, W = cam.height, cam.width
             rgb = torch.empty((H, W, 3), dtype=torch.float32, device=attrs.device)
             aux = torch.empty((5, H, W), dtype=torch.float32, device=attrs.device)
-            _after_last_backward(renderer, torch.cuda.current_stream(renderer.device))
             mgs_render_checked(renderer.ws, scene, cam, opts, rgb, aux)
         except Exception:
             mgs_unload_scene(scene)
@@ -83,16 +74,10 @@ class RenderFn(torch.autograd.Function):
         dev = aux.device
         d_attrs = torch.empty(ctx.attrs_shape, dtype=torch.float32, device=dev)
         d_mlp = torch.empty(MLP_GRAD_SIZE, dtype=torch.float32, device=dev) if ctx.n_mlp else None
-        stream = torch.cuda.current_stream(dev)
         try:
-            _after_last_backward(ctx.renderer, stream)
             mgs_render_backward(ctx.renderer.ws, ctx.scene, ctx.cam, ctx.opts, g.contiguous(), aux,
                                 d_attrs, d_mlp)
-            if ctx.borrowed:
-                done = torch.cuda.Event()
-                done.record(stream)
-                ctx.renderer._backward_done = (stream, done)
-            else:   # the library frees the scene's memory
+            if not ctx.borrowed:   # the library frees the scene's memory
                 torch.cuda.synchronize(dev)
         finally:
             mgs_unload_scene(ctx.scene)

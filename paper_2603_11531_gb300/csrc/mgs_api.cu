@@ -115,6 +115,8 @@ struct mgs_workspace_s {
     const uint32_t *last_perm = nullptr;   // storage -> caller order of the last scene
     uint64_t grow_hint = 0;  // pairs needed by an overflowed render
     uint64_t generation = 0; // bumped whenever a scratch buffer is reallocated
+    cudaEvent_t bwd_done = nullptr;   // recorded after the last backward pass
+    bool bwd_pending = false;         // a later call may have to wait for bwd_done
     bool timing = false;
     std::vector<cudaEvent_t> event_pool;
     std::vector<std::array<cudaEvent_t, kStageEvents>> pending;  // per timed render
@@ -232,6 +234,49 @@ uint64_t default_pairs(int64_t n) {
     return p < (1u << 20) ? (1u << 20) : p;
 }
 
+// A training step's backward pass returns while its kernels still use the
+// workspace, and what a program calls next may run on another stream (a preview
+// beside the training stream).  Every call that reads or writes the workspace's
+// buffers on a stream therefore first orders that stream after the last backward
+// pass.  The stream's handle says nothing about this (a destroyed stream's handle is
+// handed out again, and the per-thread default stream is another one in every
+// thread), so the wait is enqueued whichever stream it is: about 1 us of host time.
+cudaError_t order_after_backward(mgs_workspace_s *w, cudaStream_t stream) {
+    if (!w->bwd_pending) return cudaSuccess;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(stream, &cap);
+    if (e != cudaSuccess) return e;
+    if (cap == cudaStreamCaptureStatusNone) return cudaStreamWaitEvent(stream, w->bwd_done, 0);
+    // a graph cannot hold a wait for work outside it: the host waits before the capture goes on
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if ((e = cudaThreadExchangeStreamCaptureMode(&mode)) != cudaSuccess) return e;
+    e = cudaEventSynchronize(w->bwd_done);
+    const cudaError_t er = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) w->bwd_pending = false;
+    return e != cudaSuccess ? e : er;
+}
+
+// The same, and the host waits for the stream.
+cudaError_t sync_after_backward(mgs_workspace_s *w, cudaStream_t stream) {
+    cudaError_t e = order_after_backward(w, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    if (e == cudaSuccess) w->bwd_pending = false;
+    return e;
+}
+
+// After the last launch of a backward pass.  Inside a capture nothing runs yet:
+// ordering the graph's launches is the program's.
+cudaError_t mark_backward(mgs_workspace_s *w, cudaStream_t stream) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(stream, &cap);
+    if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) return e;
+    if (!w->bwd_done &&
+        (e = cudaEventCreateWithFlags(&w->bwd_done, cudaEventDisableTiming)) != cudaSuccess)
+        return e;
+    if ((e = cudaEventRecord(w->bwd_done, stream)) == cudaSuccess) w->bwd_pending = true;
+    return e;
+}
+
 // Backward request: when non-null, render_impl builds the frame's records and
 // tile lists and then runs the adjoint kernels instead of the rasteriser.
 struct BackwardIO {
@@ -308,7 +353,8 @@ mgs_status render_impl(mgs_workspace w, mgs_scene s, const mgs_camera *cam,
     }
 
     std::array<cudaEvent_t, kStageEvents> ev{};
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = order_after_backward(w, stream);
+    if (e != cudaSuccess) return cuda_fail(e, "order after the backward pass");
     if (w->timing) {
         for (auto &x : ev) {
             if (w->event_pool.empty()) {
@@ -396,6 +442,7 @@ mgs_status render_impl(mgs_workspace w, mgs_scene s, const mgs_camera *cam,
         cudaEventRecord(ev[6], stream);
         w->pending.push_back(ev);
     }
+    if (bwd && (e = mark_backward(w, stream)) != cudaSuccess) return cuda_fail(e, "backward event");
     w->last_tiles = T;
     w->last_perm = s->perm;
     return MGS_OK;
@@ -693,6 +740,7 @@ mgs_status mgs_workspace_destroy(mgs_workspace w) {
     for (auto &q : w->pending)
         for (auto x : q) cudaEventDestroy(x);
     for (auto x : w->event_pool) cudaEventDestroy(x);
+    if (w->bwd_done) cudaEventDestroy(w->bwd_done);
     delete w;
     return MGS_OK;
 }
@@ -714,7 +762,8 @@ mgs_status mgs_workspace_sync(mgs_workspace w, mgs_stream stream_, int64_t *pair
     if (!w) return fail(MGS_ERR_INVALID_ARG, "workspace is NULL");
     DeviceGuard g(w->ctx->device);
     // the status is read and reset in stream order: one wait for everything
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = order_after_backward(w, stream);
+    if (e != cudaSuccess) return cuda_fail(e, "order after the backward pass");
     if (w->status) {
         e = cudaMemcpyAsync(w->status_host, w->status, sizeof(DevStatus), cudaMemcpyDeviceToHost, stream);
         if (e != cudaSuccess) return cuda_fail(e, "status read");
@@ -722,6 +771,7 @@ mgs_status mgs_workspace_sync(mgs_workspace w, mgs_stream stream_, int64_t *pair
         if (e != cudaSuccess) return cuda_fail(e, "status reset");
     }
     if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return cuda_fail(e, "stream synchronize");
+    w->bwd_pending = false;
     if (pairs_out) *pairs_out = 0;
     if (!w->status) return MGS_OK;
     const DevStatus h = *w->status_host;
@@ -748,7 +798,7 @@ mgs_status mgs_workspace_stage_times(mgs_workspace w, mgs_stream stream_, double
     cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
     if (!w || !ms || !frames) return fail(MGS_ERR_INVALID_ARG, "NULL argument");
     DeviceGuard g(w->ctx->device);
-    cudaError_t e = cudaStreamSynchronize(stream);
+    cudaError_t e = sync_after_backward(w, stream);
     if (e != cudaSuccess) return cuda_fail(e, "stream synchronize");
     for (int k = 0; k < kStageEvents - 1; ++k) ms[k] = 0.0;
     *frames = (int64_t)w->pending.size();
@@ -836,7 +886,7 @@ mgs_status mgs_frame_stats(mgs_workspace w, mgs_stream stream_, int64_t *visible
     *visible = *pairs = *fp32_sum_tiles = 0;
     if (!w->status || w->last_tiles == 0) return fail(MGS_ERR_INVALID_ARG, "no render yet");
     DeviceGuard g(w->ctx->device);
-    cudaError_t e = cudaStreamSynchronize(stream);
+    cudaError_t e = sync_after_backward(w, stream);
     if (e != cudaSuccess) return cuda_fail(e, "stream synchronize");
     DevStatus h;
     if ((e = cudaMemcpy(&h, w->status, sizeof h, cudaMemcpyDeviceToHost)) != cudaSuccess)
@@ -854,7 +904,7 @@ mgs_status mgs_tile_lists(mgs_workspace w, mgs_stream stream_, int64_t *n_tiles,
     *n_tiles = *n_pairs = 0;
     if (!w->status || w->last_tiles == 0) return fail(MGS_ERR_INVALID_ARG, "no render yet");
     DeviceGuard g(w->ctx->device);
-    cudaError_t e = cudaStreamSynchronize(stream);
+    cudaError_t e = sync_after_backward(w, stream);
     if (e != cudaSuccess) return cuda_fail(e, "stream synchronize");
     DevStatus h;
     if ((e = cudaMemcpy(&h, w->status, sizeof h, cudaMemcpyDeviceToHost)) != cudaSuccess)
