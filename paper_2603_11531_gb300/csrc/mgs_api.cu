@@ -7,6 +7,7 @@
 #include <cstring>
 #include <string>
 #include <array>
+#include <atomic>
 #include <vector>
 
 #include "mgs_internal.cuh"
@@ -70,6 +71,11 @@ struct mgs_ctx_s {
 };
 
 struct mgs_scene_s {
+    // never given twice: a handle's address is, once its scene is unloaded
+    const uint64_t id = [] {
+        static std::atomic<uint64_t> last{0};
+        return ++last;
+    }();
     mgs_ctx ctx = nullptr;
     int64_t n = 0;
     int precision = MGS_PREC_FP32;
@@ -468,6 +474,7 @@ uint64_t mgs::workspace_generation(mgs_workspace w) { return w->generation; }
 int mgs::ctx_device(mgs_ctx c) { return c->device; }
 int mgs::ctx_sm_count(mgs_ctx c) { return c->sm_count; }
 int64_t mgs::scene_size(mgs_scene s) { return s->n; }
+uint64_t mgs::scene_id(mgs_scene s) { return s->id; }
 mgs_ctx mgs::scene_ctx(mgs_scene s) { return s->ctx; }
 
 extern "C" {

@@ -346,6 +346,7 @@ uint64_t workspace_generation(mgs_workspace w);
 int ctx_device(mgs_ctx c);
 int ctx_sm_count(mgs_ctx c);
 int64_t scene_size(mgs_scene s);
+uint64_t scene_id(mgs_scene s);   // unlike the handle, never given to another scene
 mgs_ctx scene_ctx(mgs_scene s);
 cudaError_t launch_raster(const RenderArgs &a, cudaStream_t stream);
 // Persistent rasteriser over the tiles of `nviews` views (views_dev and

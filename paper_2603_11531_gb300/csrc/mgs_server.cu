@@ -25,10 +25,12 @@
 // tile lists: alone or in a mix it is the same up to FP32 rounding of the
 // accumulation order.
 #include <algorithm>
+#include <array>
 #include <chrono>
 #include <condition_variable>
 #include <cstring>
 #include <deque>
+#include <map>
 #include <mutex>
 #include <thread>
 #include <unordered_map>
@@ -51,10 +53,17 @@ enum { kQueued = 0, kRunning = 1, kDone = 2 };
 // when several are admitted at once; larger views fill the GPU alone.
 constexpr int kSmallTiles = 2048;
 constexpr int kGraphsPerSlot = 16;
+constexpr size_t kPairsEntries = 4096;   // remembered pair counts (scene, size)
+
+// What a captured graph and a remembered pair count belong to, in full: launch
+// grids and addresses inside the workspace follow from the scene's size and kind.
+using ViewKey = std::array<uint64_t, 2>;    // scene, width | height
+using GraphKey = std::array<uint64_t, 5>;   // view, use_mlp | residual, flags, what is captured
 
 struct Request {
     int64_t ticket = 0;
     mgs_scene scene = nullptr;
+    uint64_t scene_id = 0;
     mgs_camera cam{};
     mgs_render_opts opts{};
     float *out = nullptr;
@@ -69,7 +78,7 @@ struct Request {
 // single-view rasteriser when `raster`), with the nodes whose arguments
 // depend on the camera and the output.
 struct SlotGraph {
-    uint64_t key = 0;
+    GraphKey key{};             // no scene has id 0
     uint64_t gen = 0;           // workspace buffer generation it was captured with
     uint64_t last_use = 0;
     cudaGraph_t graph = nullptr;
@@ -118,7 +127,7 @@ struct mgs_server_s {
     uint64_t clock = 0;
     bool stop = false;
     bool graphs = true;
-    std::unordered_map<uint64_t, uint64_t> pairs_cache;  // (scene, size) -> pairs
+    std::map<ViewKey, uint64_t> pairs_cache;  // pairs of the last such view
     std::thread worker;
 
     void run();
@@ -131,16 +140,14 @@ struct mgs_server_s {
 
 namespace {
 
-uint64_t cache_key(mgs_scene s, int w, int h) {
-    return (reinterpret_cast<uint64_t>(s) * 1000003ull) ^ ((uint64_t)w << 32) ^ (uint64_t)h;
+ViewKey view_key(const Request &rq) {
+    return {rq.scene_id, (uint64_t)(uint32_t)rq.cam.width << 32 | (uint32_t)rq.cam.height};
 }
 
-uint64_t graph_key(const Request &rq, bool raster, bool grouped) {
-    uint64_t k = cache_key(rq.scene, rq.cam.width, rq.cam.height);
-    k = k * 31ull + (uint64_t)rq.opts.use_mlp;
-    k = k * 31ull + (uint64_t)rq.opts.mlp_rgb_residual;
-    k = k * 131ull + (uint64_t)rq.opts.flags;
-    return k * 4ull + (raster ? 1ull : 0ull) + (grouped ? 2ull : 0ull);
+GraphKey graph_key(const Request &rq, bool raster, bool grouped) {
+    const ViewKey v = view_key(rq);
+    return {v[0], v[1], (uint64_t)(uint32_t)rq.opts.use_mlp << 32 | (uint32_t)rq.opts.mlp_rgb_residual,
+            (uint64_t)rq.opts.flags, (raster ? 1ull : 0ull) | (grouped ? 2ull : 0ull)};
 }
 
 int64_t estimate_bytes(int64_t n, int w, int h, uint64_t pairs, int sm_count) {
@@ -195,7 +202,7 @@ mgs_status launch_view(mgs_server_s *S, Slot &sl, Request &rq, bool raster, bool
         return st;
     };
     if (!S->graphs) return direct();
-    const uint64_t key = graph_key(rq, raster, grouped);
+    const GraphKey key = graph_key(rq, raster, grouped);
     const uint64_t gen = workspace_generation(sl.ws);
     SlotGraph *hit = nullptr;
     for (SlotGraph &g : sl.graphs)
@@ -221,7 +228,7 @@ mgs_status launch_view(mgs_server_s *S, Slot &sl, Request &rq, bool raster, bool
             return MGS_OK;
         }
         cudaGetLastError();
-        hit->key = 0;   // unusable: recapture below
+        hit->key = {};   // unusable: recapture below
     }
     // capture this key's graph (the workspace is sized first, outside capture)
     {
@@ -299,7 +306,8 @@ void mgs_server_s::run() {
                 Slot &sl = slots[si];
                 Request &rq = reqs[sl.ticket];
                 const uint64_t need = sl.status_host->last_pairs;
-                pairs_cache[cache_key(rq.scene, rq.cam.width, rq.cam.height)] = need;
+                if (pairs_cache.size() >= kPairsEntries) pairs_cache.clear();
+                pairs_cache[view_key(rq)] = need;
                 if (q != cudaSuccess || (sl.status_host->overflow & kStatusMmaTimeout)) {
                     rq.result = q != cudaSuccess ? MGS_ERR_CUDA : MGS_ERR_TIMEOUT;
                     rq.state = kDone;
@@ -357,7 +365,7 @@ void mgs_server_s::run() {
                         free_slot = k;
                 if (free_slot < 0) break;
                 const int64_t n = scene_size(rq.scene);
-                auto it = pairs_cache.find(cache_key(rq.scene, rq.cam.width, rq.cam.height));
+                auto it = pairs_cache.find(view_key(rq));
                 uint64_t pairs = it != pairs_cache.end() ? it->second + it->second / 8 + 1024
                                                          : (uint64_t)std::max<int64_t>(48 * n, 1 << 20);
                 pairs = std::max(pairs, rq.pairs_hint);
@@ -587,6 +595,7 @@ mgs_status mgs_server_submit(mgs_server S, mgs_scene scene, const mgs_camera *ca
     if (validate_camera(cam) != MGS_OK) return MGS_ERR_INVALID_ARG;
     Request rq;
     rq.scene = scene;
+    rq.scene_id = scene_id(scene);
     rq.cam = *cam;
     rq.opts = *opts;
     rq.out = out_rgb;
