@@ -98,11 +98,18 @@ struct BwdRaster {
     float4 ring[kBwdWarps][3][kBwdRing];
 };
 
-// How a batch treats the pixels: kFast (every constant finite, no opacity above
-// 0.99: an excluded pixel's alpha is 0 and so is everything it adds), kClamped
-// (some opacity above 0.99) and kGuarded (a non-finite weight, colour or pixel
-// constant: excluded pixels are skipped, so that they add nothing).
+// How a batch treats the pixels: kFast (every product of an excluded pixel finite,
+// no opacity above 0.99: its alpha is 0 and so is everything it adds), kClamped
+// (some opacity above 0.99) and kGuarded (a pixel constant is not finite, or some
+// candidate's weight or colour is so large, or not finite, that its products with
+// the block's pixel constants may leave the FP32 range, where 0 times them is NaN:
+// excluded pixels are skipped, so that they add nothing).
 enum BwdMode { kFast, kClamped, kGuarded };
+constexpr float kSafeProduct = 1e38f;   // FP32's largest number is 3.4e38
+
+__device__ __forceinline__ float warp_max(float v) {   // v >= 0, or NaN
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
 
 // One batch: lane = one candidate, looping over the warp's 8x8 block at (bx0,
 // by0); adds the candidate's ten partials to its gradient record.
@@ -274,6 +281,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_raster_bwd(RenderArgs args,
     // this lane's pixel pair: constants from the forward's (A, B, T) and dL/dC,
     // with k_A = (1 - T) / B and r = A / B (all zero without coverage)
     bool finite = true;
+    float k_lane = 0.f, kr_lane = 0.f, tg_lane = 0.f;
     {
         const int64_t HW = (int64_t)cam.width * cam.height;
         const int py = by0 + (lane >> 2), x0 = bx0 + 2 * (lane & 3);
@@ -303,12 +311,18 @@ __global__ void __launch_bounds__(kBwdThreads) k_raster_bwd(RenderArgs args,
             }
 #pragma unroll
             for (int e = 0; e < 5; ++e) finite &= isfinite(k[e][h]);
+            k_lane = fmaxf(k_lane, fabsf(k[0][h]) + fabsf(k[1][h]) + fabsf(k[2][h]));
+            kr_lane = fmaxf(kr_lane, fabsf(k[3][h]));
+            tg_lane = fmaxf(tg_lane, fabsf(k[4][h]));
         }
         sm.px0[warp][lane] = make_float4(k[0][0], k[0][1], k[1][0], k[1][1]);
         sm.px1[warp][lane] = make_float4(k[2][0], k[2][1], k[3][0], k[3][1]);
         sm.px2[warp][lane] = make_float2(k[4][0], k[4][1]);
     }
     const bool px_finite = __all_sync(0xffffffffu, finite);
+    // block maxima of |k_A G_r| + |k_A G_g| + |k_A G_b|, |k_A G.r| and |T G.(c_bg - r)|
+    // (finite non-negative floats order as unsigned integers)
+    const float k_max = warp_max(k_lane), kr_max = warp_max(kr_lane), tg_max = warp_max(tg_lane);
     const float bx = (float)bx0 + 4.0f, by = (float)by0 + 4.0f;
     const float kLogClamp = -0.014499569695115089f;   // log2(0.99)
     float4(*ring)[kBwdRing] = sm.ring[warp];
@@ -320,7 +334,12 @@ __global__ void __launch_bounds__(kBwdThreads) k_raster_bwd(RenderArgs args,
         bool special = false, clamp = false;
         if (active) {
             const float4 b = ring[1][slot], c = ring[2][slot];
-            special = !(fabsf(b.w) + fabsf(c.x) + fabsf(c.y) + fabsf(c.z) < INFINITY);
+            // bounds u and w u + tg of every excluded pixel (1 - a = 1 there), and
+            // fails for a NaN
+            const float c_max = fmaxf(fmaxf(fabsf(c.x), fabsf(c.y)), fabsf(c.z));
+            const float u_max = fmaf(k_max, c_max, kr_max);
+            special = !(fmaf(fmaxf(fabsf(b.w), 1.0f), u_max, tg_max) < kSafeProduct &&
+                        fabsf(b.w) + fabsf(c.x) + fabsf(c.y) + fabsf(c.z) < INFINITY);
             clamp = !(b.y <= kLogClamp);
         }
         if (!px_finite || __any_sync(0xffffffffu, special))
