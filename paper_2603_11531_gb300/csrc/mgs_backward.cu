@@ -378,8 +378,10 @@ __global__ void __launch_bounds__(kBwdThreads) k_raster_bwd(RenderArgs args,
             const float w = -b.z, o = exp2f(b.y);
             const float iw = 1.0f / w;
             ring[0][pos] = a;
-            // 1 / o (0 when o = 0: no opacity gradient then); colour c = (-w c) / (-w)
-            ring[1][pos] = make_float4(b.x, b.y, o > 0.0f ? 1.0f / o : 0.0f, w);
+            // 1 / o (0 when o = 0: no opacity gradient then; nor below FP32's smallest
+            // normal number, where alpha is flushed to 0 and 1 / o may be infinite);
+            // colour c = (-w c) / (-w)
+            ring[1][pos] = make_float4(b.x, b.y, o >= 1.1754943508222875e-38f ? 1.0f / o : 0.0f, w);
             ring[2][pos] = make_float4(-b.w * iw, -c.x * iw, -c.y * iw, __uint_as_float(gid));
         }
         __syncwarp();
