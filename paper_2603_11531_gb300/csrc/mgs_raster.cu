@@ -24,13 +24,12 @@
 // No atomics, no sort: every pixel belongs to one quad, and a tile's list is
 // accumulated in whatever order binning stored it.
 //
-// The FMA sums stop updating T once it cannot matter: when every lane of a warp holds
-// a partial product of at most 2^-12 for each of its pixels, T <= 2^-48, so
-// 1 - T is 1 in FP32 and T c_bg is below 2^-40 for |c_bg| <= 256 (a larger
-// background keeps the updates, and so does the aux output, which returns T).
-// The frozen value stays an upper bound of T.  The tensor-core sums, whose lists are
-// the longer ones, stop at partial products of 2^-8 and |c_bg| <= 4: T <= 2^-32 and
-// T c_bg <= 2^-30, below half a unit in the last place of any colour above 2^-6.
+// T stops being updated where no further update can change a bit of the image: a
+// lane's partial product only shrinks, so once every lane of a warp holds at most
+// 2^-38 for each of its pixels, the product over a quad is at most 2^-152, which FP32
+// rounds to 0, as it does the product of anything smaller.  With a background of zeros
+// T c_bg is 0 whatever T is, and 2^-8 suffices: T <= 2^-32, so that 1 - T rounds to 1.
+// A NaN stays NaN, updated or not.  The aux output returns T and keeps the updates.
 #include "mgs_internal.cuh"
 
 namespace mgs {
@@ -38,10 +37,8 @@ namespace {
 
 constexpr int kThreads = 128;
 constexpr int kWarps = kThreads / 32;
-constexpr float kFrozenT = 0.000244140625f;   // 2^-12
-constexpr float kMaxFrozenBg = 256.0f;
-constexpr float kFrozenTcT = 0.00390625f;     // 2^-8, tensor-core sums
-constexpr float kMaxFrozenTcBg = 4.0f;
+constexpr float kZeroT = 3.637978807091713e-12f;   // 2^-38: T is 0
+constexpr float kOneMinusT = 0.00390625f;          // 2^-8: 1 - T is 1
 constexpr int kFreezeEvery = 128;             // list entries between two checks
 constexpr float kLogClamp = -0.014499569695115089f;   // log2(0.99)
 
@@ -139,13 +136,21 @@ __device__ __forceinline__ void accumulate(const ulonglong2 (*wb)[kRingF], int k
     }
 }
 
-// Does every lane hold partial products of at most `bound`?
-__device__ __forceinline__ bool all_frozen(float m, float bound) {
-    return __all_sync(0xffffffffu, m <= bound);
+// Every lane's partial products at most this: T no longer matters (see above).
+__device__ __forceinline__ bool zero_bg(const RenderArgs &args) {
+    return args.bg[0] == 0.0f && args.bg[1] == 0.0f && args.bg[2] == 0.0f;
 }
-
-__device__ __forceinline__ bool may_freeze(const RenderArgs &args, float max_bg) {
-    return fmaxf(fmaxf(fabsf(args.bg[0]), fabsf(args.bg[1])), fabsf(args.bg[2])) <= max_bg;
+__device__ __forceinline__ bool all_frozen(const RenderArgs &args, float m) {
+    return __all_sync(0xffffffffu, m <= (zero_bg(args) ? kOneMinusT : kZeroT));
+}
+// May T stop being updated?  0 c_bg is 0 for a finite background only.  The depth image's
+// lists rarely reach 2^-38 and only pay for the question (300k at 1280x720: 0.393 ms with
+// it, 0.388 without; 0.379 with a background of zeros, which freezes at 2^-8).
+template <bool kAux, bool kDepth>
+__device__ __forceinline__ bool may_freeze(const RenderArgs &args) {
+    if (kAux) return false;
+    if (kDepth) return zero_bg(args);
+    return fmaxf(fmaxf(fabsf(args.bg[0]), fabsf(args.bg[1])), fabsf(args.bg[2])) < INFINITY;
 }
 
 // Writes one pixel's outputs from its sums.
@@ -257,7 +262,7 @@ __device__ __forceinline__ void raster_tile(const RenderArgs &args, int tile, Fm
     int head = 0, count = 0;   // queued candidates: ring slots [head, head + count) mod kRingF
     int clamp_left = 0;        // queued candidates up to the last whose opacity exceeds 0.99
     bool live = true;          // T is still updated
-    const bool freeze = !kAux && may_freeze(args, kMaxFrozenBg);
+    const bool freeze = may_freeze<kAux, false>(args);
     auto group = [&]() {
         const int k = head + t;
         if (live) {
@@ -316,9 +321,8 @@ __device__ __forceinline__ void raster_tile(const RenderArgs &args, int tile, Fm
                 float x, y;
                 upk(S.T[p], x, y);
                 m = fmaxf(m, fmaxf(x, y));
-                if (!(x <= 1.0f && y <= 1.0f)) m = 1.0f;   // NaN: keep updating
             }
-            live = !all_frozen(m, kFrozenT);
+            live = !all_frozen(args, m);
         }
         __syncwarp();
     }
@@ -380,13 +384,13 @@ __device__ __forceinline__ void raster_tile(const RenderArgs &args, int tile, Fm
 // A / B and is divided out here).  T stays in FP32 FMAs.  Tiles listing a Gaussian
 // outside that scale's range (kTileWide) are rasterised by the FMA tile code.
 //
-// Bound: instruction issue (83 % of the slots used; a packed FP32x2 operation takes
-// two), so the time follows the instructions per pixel: without T's two FMAs where T
-// is frozen, and with the weight fragment read by one ldmatrix instead of two 16-bit
-// loads and a merge, 600k Gaussians at 1600x1063 take 0.814 ms (0.863 before; either
-// change alone 0.841 and 0.866), depth of 300k at 1280x720 0.381 ms (0.388).  Lists
-// too short to freeze pay about 1 us per launch for the choice (50k at 640x480: 34.7
-// against 33.8 us).  Two lanes per record instead of one (cp.async into shared memory)
+// Bound: instruction issue (78 % of the slots used at 600k Gaussians, 1600x1063; a packed
+// FP32x2 operation takes two), so the time follows the instructions per pixel: without
+// T's two FMAs where T is frozen, and with the weight fragment read by one ldmatrix
+// instead of two 16-bit loads and a merge, that frame takes 0.834 ms with a background
+// and 0.810 ms on zeros (0.865 never frozen), 3M at 640x480 1.34 and 1.33 ms (1.43), 6M at
+// 3840x2160 36.9 and 36.7 ms (40.1); 50k at 640x480, whose lists are too short to
+// freeze, 34.1 us (34.2).  Two lanes per record instead of one (cp.async into shared memory)
 // saves L1 tag lookups but waits longer: 0.876 ms.
 constexpr int kChunk = 8;        // candidates per MMA (K)
 constexpr int kRing = 64;        // candidate slots per warp: eight chunks (a power of two)
@@ -512,7 +516,7 @@ __device__ __forceinline__ void raster_tile_tc(const RenderArgs &args, int tile,
 
     int head = 0, count = 0;          // unprocessed candidates: ring slots [head, head + count)
     uint64_t clamp_mask = 0;          // ring slots whose opacity exceeds 0.99
-    const bool freeze = !kAux && may_freeze(args, kMaxFrozenTcBg);
+    const bool freeze = may_freeze<kAux, kDepth>(args);
     bool live = true;                 // T is still updated
     auto chunk = [&]() {
         const bool clamp = ((clamp_mask >> head) & 0xFFull) != 0;
@@ -599,8 +603,8 @@ __device__ __forceinline__ void raster_tile_tc(const RenderArgs &args, int tile,
         if (freeze && live && ((base - start) & (kFreezeEvery - 1)) == kFreezeEvery - 32) {
             float m = T[0];
 #pragma unroll
-            for (int k = 1; k < 8; ++k) m = T[k] <= m ? m : T[k];   // NaN: keep updating
-            live = !all_frozen(m, kFrozenTcT);
+            for (int k = 1; k < 8; ++k) m = fmaxf(m, T[k]);
+            live = !all_frozen(args, m);
         }
         __syncwarp();
     }
