@@ -616,7 +616,7 @@ __device__ __forceinline__ Share plan_shares(const uint32_t *__restrict__ cost, 
 }
 
 // The same share, as k_bin_count stored it.
-__device__ __forceinline__ Share stored_share(const unsigned long long *__restrict__ plan, int groups) {
+__device__ __forceinline__ Share stored_share(const unsigned long long *plan, int groups) {
     Share sh = share_of(plan[0], groups);
     if (sh.len > 0) {
         const unsigned long long p = plan[1 + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)];
@@ -728,12 +728,14 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_bin_count(const uint2 *__res
 constexpr int64_t kOpenSectors = (int64_t)128 << 20 >> 5;
 constexpr int kLaneRun = 16;
 
+// Its CTAs may be resident while k_scan_order still runs: what that kernel or the
+// count writes is read through plain pointers, so that no load is taken for one of
+// data that stay constant for as long as this kernel lives.
 __global__ void __launch_bounds__(kBinThreads, 2) k_bin_scatter(
     const uint2 *__restrict__ rect, int64_t n, int tiles_x, int tiles_y,
-    const uint32_t *__restrict__ cost, int groups, const unsigned long long *__restrict__ plan,
-    const uint32_t *__restrict__ offsets, const uint32_t *__restrict__ bases,
-    uint32_t *__restrict__ gids, uint64_t capacity, const DevStatus *__restrict__ status,
-    const ProjRec *__restrict__ rec, uint4 *__restrict__ wt16) {
+    const uint32_t *__restrict__ cost, int groups, const unsigned long long *plan,
+    const uint32_t *offsets, const uint32_t *bases, uint32_t *gids, uint64_t capacity,
+    const DevStatus *status, const ProjRec *__restrict__ rec, uint4 *__restrict__ wt16) {
     grid_wait();
     extern __shared__ uint32_t cur_s[];
     __shared__ RowSlot queue_s[kBinThreads / 32][kQueue];
@@ -821,7 +823,9 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_bin_scatter(
 //     accumulator (and the wide-Gaussian flag) for the next frame;
 //   * carries each tile's kTileWide flag from tile_count[] into its order
 //     entry.
-__global__ void __launch_bounds__(kScanThreads) k_scan_order(const uint32_t *__restrict__ count,
+// It may be resident while the count still writes tile_count: a plain pointer, as in
+// k_bin_scatter.
+__global__ void __launch_bounds__(kScanThreads) k_scan_order(const uint32_t *count,
                                                              uint32_t *__restrict__ offsets,
                                                              uint32_t *__restrict__ order, int T,
                                                              uint64_t capacity, DevStatus *status) {
