@@ -81,7 +81,9 @@ class RenderFn(torch.autograd.Function):
                 torch.cuda.synchronize(dev)
         finally:
             mgs_unload_scene(ctx.scene)
-            ctx.scene = None
+            # the graph may outlive this pass (a program that keeps its losses); the
+            # tensors go back to the stream that the pass runs on
+            ctx.scene = ctx.borrowed = None
         grads = [None, None, None, d_attrs.to(ctx.attrs_dtype)]
         if ctx.n_mlp:
             grads += [t.view(shp) for t, (_, shp) in zip(d_mlp.split(_SIZES), _SHAPES)]
