@@ -43,6 +43,9 @@ def _step_scene(renderer, attrs, mlp):
     if mlp:
         params = [t if t.dtype == torch.float32 and t.device == a.device and t.is_contiguous()
                   else t.detach().to(device=a.device, dtype=torch.float32).contiguous() for t in mlp]
+        # frozen biases may be columns or rows, as mgs_load_scene takes them
+        params = [t if t.ndim == len(shp) else t.detach().reshape(-1) if len(shp) == 1 else t
+                  for t, (_, shp) in zip(params, _SHAPES, strict=True)]
         blob = torch.empty(mgs_mlp_blob_bytes(), dtype=torch.uint8, device=a.device)
     return mgs_borrow_scene(renderer.ctx, a, params, blob), (a, blob)
 
