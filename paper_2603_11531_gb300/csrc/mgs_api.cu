@@ -29,6 +29,7 @@ mgs_status fail(mgs_status s, const char *fmt, ...) {
 }
 
 mgs_status cuda_fail(cudaError_t e, const char *what) {
+    cudaGetLastError();   // reported here, not by the next call's launch check
     if (e == cudaErrorMemoryAllocation)
         return fail(MGS_ERR_OOM, "%s: %s", what, cudaGetErrorString(e));
     return fail(MGS_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));

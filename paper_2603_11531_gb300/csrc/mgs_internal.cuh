@@ -35,7 +35,9 @@ cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(std::forward<A>(args))...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(std::forward<A>(args))...);
+    if (e != cudaSuccess) cudaGetLastError();   // reported here, not by the next launch's check
+    return e;
 }
 
 constexpr int kTile = 16;         // tile edge in pixels (binning granularity)
