@@ -186,6 +186,9 @@ mgs_status mgs_workspace_reserve(mgs_workspace ws, int64_t n, int32_t width,
                                  int32_t height, int64_t pairs);
 /* Device bytes held by the workspace. */
 int64_t mgs_workspace_bytes(mgs_workspace ws);
+/* 1 once a call on this workspace has been captured into a CUDA graph.  The library does
+ * not see a graph's launches: the program orders them after mgs_render_backward. */
+int32_t mgs_workspace_captured(mgs_workspace ws);
 /* Wait for `stream`, then report renders since the previous sync:
  * MGS_ERR_OVERFLOW if any ran out of tile-list capacity (the workspace is then
  * grown so that a repeat succeeds); MGS_ERR_TIMEOUT if a tensor-core MMA wait

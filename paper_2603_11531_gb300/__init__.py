@@ -41,7 +41,7 @@ MGS_ORDER_AS_GIVEN = 2
 EXPORTS = (
     "mgs_ctx_create", "mgs_ctx_destroy", "mgs_ctx_info", "mgs_load_scene",
     "mgs_borrow_scene", "mgs_mlp_blob_bytes", "mgs_unload_scene", "mgs_scene_bytes", "mgs_workspace_create", "mgs_workspace_destroy",
-    "mgs_workspace_reserve", "mgs_workspace_bytes", "mgs_workspace_sync", "mgs_render",
+    "mgs_workspace_reserve", "mgs_workspace_bytes", "mgs_workspace_captured", "mgs_workspace_sync", "mgs_render",
     "mgs_render_checked", "mgs_render_to_host", "mgs_tile_lists", "mgs_last_error",
     "mgs_version", "mgs_workspace_set_timing", "mgs_workspace_stage_times",
     "mgs_render_static", "mgs_render_backward", "mgs_render_depth", "mgs_decode_sh",
@@ -109,6 +109,7 @@ def lib():
                 "mgs_workspace_destroy": ([P], I32),
                 "mgs_workspace_reserve": ([P, I64, I32, I32, I64], I32),
                 "mgs_workspace_bytes": ([P], I64),
+                "mgs_workspace_captured": ([P], I32),
                 "mgs_workspace_sync": ([P, P, ctypes.POINTER(I64)], I32),
                 "mgs_render": ([P, P, ctypes.POINTER(mgs_camera), ctypes.POINTER(mgs_render_opts),
                                 P, P, P, P], I32),
@@ -374,6 +375,10 @@ def mgs_workspace_reserve(ws, n, width, height, pairs):
 
 def mgs_workspace_bytes(ws) -> int:
     return lib().mgs_workspace_bytes(ws)
+
+
+def mgs_workspace_captured(ws) -> bool:
+    return lib().mgs_workspace_captured(ws) != 0
 
 
 def mgs_workspace_sync(ws, stream=None, allow_overflow=False):

@@ -16,7 +16,7 @@ import torch
 
 from . import (MLP_GRAD_SIZE, Renderer, camera_struct, mgs_borrow_scene, mgs_camera, mgs_load_scene,
                mgs_mlp_blob_bytes, mgs_render_backward, mgs_render_checked, mgs_unload_scene,
-               render_opts)
+               mgs_workspace_captured, render_opts)
 from .synth import MLPWeights, f32_to_bf16_bits
 
 _SHAPES = (("w1", (64, 22)), ("b1", (64,)), ("w2", (64, 64)), ("b2", (64,)),
@@ -80,7 +80,9 @@ class RenderFn(torch.autograd.Function):
         try:
             mgs_render_backward(ctx.renderer.ws, ctx.scene, ctx.cam, ctx.opts, g.contiguous(), aux,
                                 d_attrs, d_mlp)
-            if not ctx.borrowed:   # the library frees the scene's memory
+            # the library frees a loaded scene's memory; and the launch of a graph that
+            # holds a render of this renderer cannot be ordered after this pass
+            if not ctx.borrowed or mgs_workspace_captured(ctx.renderer.ws):
                 torch.cuda.synchronize(dev)
         finally:
             mgs_unload_scene(ctx.scene)

@@ -124,6 +124,7 @@ struct mgs_workspace_s {
     uint64_t generation = 0; // bumped whenever a scratch buffer is reallocated
     cudaEvent_t bwd_done = nullptr;   // recorded after the last backward pass
     bool bwd_pending = false;         // a later call may have to wait for bwd_done
+    bool captured = false;            // some graph holds launches on these buffers
     bool timing = false;
     std::vector<cudaEvent_t> event_pool;
     std::vector<std::array<cudaEvent_t, kStageEvents>> pending;  // per timed render
@@ -249,10 +250,11 @@ uint64_t default_pairs(int64_t n) {
 // handed out again, and the per-thread default stream is another one in every
 // thread), so the wait is enqueued whichever stream it is: about 1 us of host time.
 cudaError_t order_after_backward(mgs_workspace_s *w, cudaStream_t stream) {
-    if (!w->bwd_pending) return cudaSuccess;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(stream, &cap);
     if (e != cudaSuccess) return e;
+    w->captured |= cap != cudaStreamCaptureStatusNone;
+    if (!w->bwd_pending) return cudaSuccess;
     if (cap == cudaStreamCaptureStatusNone) return cudaStreamWaitEvent(stream, w->bwd_done, 0);
     // a graph cannot hold a wait for work outside it: the host waits before the capture goes on
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -764,6 +766,8 @@ mgs_status mgs_workspace_reserve(mgs_workspace w, int64_t n, int32_t width, int3
 }
 
 int64_t mgs_workspace_bytes(mgs_workspace w) { return w ? ws_bytes(w) : 0; }
+
+int32_t mgs_workspace_captured(mgs_workspace w) { return w && w->captured ? 1 : 0; }
 
 mgs_status mgs_workspace_sync(mgs_workspace w, mgs_stream stream_, int64_t *pairs_out) {
     cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
