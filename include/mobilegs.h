@@ -200,11 +200,11 @@ mgs_status mgs_workspace_sync(mgs_workspace ws, mgs_stream stream,
 
 /* Per-stage device timing (the runtime breakdown the paper reports in
  * Fig. 2 and Fig. 6).  While enabled, every render on the workspace records
- * CUDA events on its stream around (0) preprocessing incl. the MLP, the four
- * parts of binning -- (1) nothing any more (the work plan is part of the
- * count), (2) the work plan and tile count, (3) the tile scan and order,
- * (4) the scatter of the lists -- and (5) rasterisation (the sorted
- * comparator's sort and blend; the backward pass's adjoint). */
+ * CUDA events on its stream around (0) preprocessing incl. the MLP and the
+ * work plan's group costs, (2) the binning's work plan and tile count, (3) the
+ * tile scan and order, (4) the scatter of the lists and (5) rasterisation (the
+ * sorted comparator's sort and blend; the backward pass's adjoint).  Entry (1)
+ * holds no work: it reads the time between two events. */
 mgs_status mgs_workspace_set_timing(mgs_workspace ws, int32_t enable);
 /* Wait for `stream`; ms[0..5] = summed stage times in milliseconds of the
  * renders timed since the previous call, *frames = their number.  Resets. */

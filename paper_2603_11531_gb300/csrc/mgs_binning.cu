@@ -286,8 +286,6 @@ __device__ __forceinline__ bool row_tiles(float mx, float my, float l11, float l
     return true;
 }
 
-// Plan cost of a rectangle row: kRowCost plus its width, summed per group by
-// preprocessing.
 // Cost of a group in the work plan beyond its rows: a fixed charge for
 // visiting it (loading its 32 rectangles, the scans and the row split), so
 // that shares over sparse stretches of the scene (many Gaussians with one
@@ -725,6 +723,7 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_bin_count(const uint2 *__res
 // Scatter, lane by lane / spread: 6M at 3840x2160 (158 MB of sectors) 6.73 / 6.21 ms,
 // 1M 2.69 / 2.65 and 300k 0.363 / 0.358 at that size; 3M at 2560x1440 (70 MB)
 // 1.16 / 1.27, 6M at 1920x1080 (40 MB) 1.29 / 1.96, 600k at 1600x1063 0.121 / 0.129.
+// The line lies at the size of GB300's L2 (129 MB); between 70 and 158 MB it was not measured.
 constexpr int64_t kOpenSectors = (int64_t)128 << 20 >> 5;
 constexpr int kLaneRun = 16;
 
@@ -936,11 +935,12 @@ cudaError_t launch_binning(const RenderArgs &a, int sm_count, uint32_t *scratch,
     const int T = tx * ty;
     const int CL = bin_ctas(a.n, sm_count);   // the scratch's layout
     // Views prepared side by side fill the chip between them, so each takes at most
-    // half as many CTAs: less per-CTA work (clearing and scanning T counts).  A burst of
-    // twelve views of 160k Gaussians: 1.087 ms with one CTA per SM and view, 1.078 with
-    // one per two SMs in a group of views, 1.066 where the lone views of a busy server
-    // do the same; a third and a quarter of the SMs are slower (1.071 and 1.108 where
-    // half took 1.053).
+    // half as many CTAs: less per-CTA work (clearing and scanning T counts, summing the
+    // plan).  A burst of twelve views of 160k Gaussians: 1.087 ms with one CTA per SM and
+    // view, 1.078 with one per two SMs in a group of views, 1.066 where the lone views of
+    // a busy server do the same; a third and a quarter of the SMs are slower (1.071 and
+    // 1.108 where half took 1.053).  This is what the plan inside the count had cost the
+    // burst (1.06 with a plan kernel of its own), not a gain over it.
     const int C = grouped ? std::min(CL, std::max(sm_count / 2, 1)) : CL;
     const int64_t groups = (a.n + 31) / 32;
     uint32_t *bases = scratch;

@@ -742,13 +742,21 @@ __device__ __forceinline__ void accumulate_wide(const ulonglong2 (*wb)[32], int 
     }
 }
 
-// FMA tile code of wide tiles in the tensor-core kernels (two warps); warp w owns the 16x8 pixel
-// block of rows 8w..8w+7, lane l the four pixels (4 (l & 3) .. +3, l >> 2) of
-// that block.  Each warp streams the tile's list on its own (no block-wide
-// barrier): 32 entries at a time, one per lane (the next 32 are fetched while
-// the current ones are accumulated), are tested against the warp's block,
-// compacted into the warp's shared-memory buffer (ballot) and accumulated by
-// all lanes.
+// FMA tile code inside the tensor-core kernels: wide tiles of FP16 views and every tile
+// of an FP32 view in the batched kernel.  Two warps; warp w owns the 16x8 pixel block of
+// rows 8w..8w+7, lane l the four pixels (4 (l & 3) .. +3, l >> 2) of that block.  Each
+// warp streams the tile's list on its own (no block-wide barrier): 32 entries at a time,
+// one per lane (the next 32 are fetched while the current ones are accumulated), are
+// tested against the warp's block, compacted into the warp's shared-memory buffer
+// (ballot) and accumulated by all lanes.
+//
+// raster_tile is 1.27 times as fast where it is a kernel's only code, but its eight
+// pixels per lane cost the code around it more than wide tiles, which are rare, can give
+// back: in k_raster_tc, where the tensor-core tiles then took 0.861 ms at 600k Gaussians,
+// 1600x1063, they took 0.96 ms beside it inlined and 0.876 ms with it out of line.  In
+// k_raster_batch it takes 128 registers instead of 112 and gains nothing: bursts of twelve
+// FP32 views of 40k to 160k Gaussians 1.238 ms against 1.239 ms here, of 150k to 600k
+// 4.05 against 4.08 ms.
 template <bool kAux, bool kCount, bool kDepth = false>
 __device__ __forceinline__ void raster_tile_wide(const RenderArgs &args, int tile,
                                             ulonglong2 (*buf)[kDepth ? 6 : 5][32]) {
