@@ -286,6 +286,9 @@ __device__ __forceinline__ bool row_tiles(float mx, float my, float l11, float l
     return true;
 }
 
+// Plan cost of a rectangle row: kRowCost plus its width (mgs_internal.cuh), summed per
+// group by preprocessing.
+
 // Cost of a group in the work plan beyond its rows: a fixed charge for
 // visiting it (loading its 32 rectangles, the scans and the row split), so
 // that shares over sparse stretches of the scene (many Gaussians with one
