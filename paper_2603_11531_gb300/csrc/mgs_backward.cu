@@ -253,12 +253,13 @@ __device__ __forceinline__ void bwd_batch(const BwdRaster &sm, int warp, int slo
 //
 // Bound: the FP32 FMA pipe (19 packed operations of two cycles each per pixel
 // pair, 0.36 ms for the pairs below) and issue.  Measured at 300k Gaussians,
-// 1296x840 (12 M (block, Gaussian) pairs): 0.67 ms, 0.54 G instructions, FMA
+// 1296x840 (12 M (block, Gaussian) pairs): 0.69 ms, 0.53 G instructions, FMA
 // pipe 60 % busy.  The layout it replaced (lane = four pixels of a 16x8 block,
 // ten partials per candidate reduced through shared memory, ten scalar
 // atomics) took 1.85 ms and 1.52 G instructions; at 30k, 333x251 (336 tiles)
 // 0.27 against 0.06 ms, there also because the lists are split over CTAs.
-// Variants that were slower: 80 registers for six CTAs per SM (0.69 ms,
+// Bounding each candidate's products takes 0.01 ms of it.  Variants that were
+// slower than 0.67 ms without that: 80 registers for six CTAs per SM (0.69 ms,
 // spills), pairs unrolled by two instead of four (0.78 ms).
 __global__ void __launch_bounds__(kBwdThreads) k_raster_bwd(RenderArgs args,
                                                             const float *__restrict__ dL,
